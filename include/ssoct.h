@@ -303,6 +303,7 @@ typedef struct {
  * lateral kernel's (lag, ring slots), lag in {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}
  * up to nlambda - 1, each with lag + 2, lag + 4 and all of the workspace's
  * slots (more for smaller frames, whose frames go through the queue faster),
+ * and the default of a new plan,
  * times the FP32 and tensor-core axial forms when nlambda is 256, in the paper's order and, where the plan offers it, in the axial-first
  * order (Eq. 5 + Eq. 7 before Eq. 6, the same V; offered when the frame size
  * has the persistent lateral kernel and a width that is a multiple of 64,

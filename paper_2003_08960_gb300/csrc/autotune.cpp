@@ -127,7 +127,7 @@ extern "C" ssoct_status ssoct_autotune(ssoct_plan h, const uint16_t* frames_dev,
   // schedule (generic-path plans have none), times the axial forms this sweep
   // length has (paper order).  Schedules: lags from 1 up to what the ring
   // allows, each with the fewest slots it needs (lag + 2), two more, and the
-  // whole ring.
+  // whole ring; and the default schedule of lateral_pick.
   std::vector<Choice> cand;
   const int lags[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32};
   for (int af = 0; af <= 1; ++af)
@@ -147,6 +147,12 @@ extern "C" ssoct_status ssoct_autotune(ssoct_plan h, const uint16_t* frames_dev,
           if (valid(p, c)) cand.push_back(c);
         }
       }
+      // the plan's default, where it is none of these
+      const LateralPick d = lateral_pick(p.nl, p.sch.n_row + p.sch.n_col, p.slots_alloc);
+      const Choice c{d.lag, d.slots, tc, af};
+      bool have = !valid(p, c);
+      for (const Choice& o : cand) have = have || (o.lag == c.lag && o.slots == c.slots && o.tc == tc && o.af == af);
+      if (!have) cand.push_back(c);
     }
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return SSOCT_ECUDA;

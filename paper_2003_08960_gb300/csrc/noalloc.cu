@@ -11,8 +11,8 @@
 // path needs lives in one file-scope device array.
 //
 // The array holds the plan's tables, the L2 scratch ring and work counters of
-// the lateral kernel, and the sweep-axis intermediate, laid out exactly like a
-// plan workspace.  It has a fixed size (kNoAllocBytes), and every GPU that loads
+// the lateral kernel, and the sweep-axis intermediate: the tables and counters
+// where a plan workspace has them, then the ring and the intermediate.  It has a fixed size (kNoAllocBytes), and every GPU that loads
 // the library keeps it until the process exits.  All calls share it and it keeps
 // the last call's contents: each call rewrites the tables and zeroes the
 // counters before its kernels run, and calls that overlap on the GPU (different
@@ -21,6 +21,7 @@
 // A kernel that gives up a bounded wait leaves its error word in the array;
 // ssoct_sync on the same plan reads it (noalloc_error_word) and reports
 // SSOCT_ETIMEOUT, as it does for the workspace path.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <mutex>
@@ -83,11 +84,11 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   if (p.af_forced) return fail(p, SSOCT_EUNSUPPORTED, "the no-allocation entry point runs the paper's order");
   PaperOrderScope paper_order(p);  // an autotuned axial-first choice does not apply here
   if (p.generic) return fail(p, SSOCT_EUNSUPPORTED, "the no-allocation entry point needs a frame size of the persistent lateral kernel");
-  if (p.ws_bytes > kNoAllocBytes) {
+  if (p.noalloc_bytes > kNoAllocBytes) {
     char msg[200];
     snprintf(msg, sizeof msg,
              "this plan needs %zu bytes of device scratch; the no-allocation entry point holds at most %zu (64 MiB)",
-             p.ws_bytes, kNoAllocBytes);
+             p.noalloc_bytes, kNoAllocBytes);
     return fail(p, SSOCT_EUNSUPPORTED, msg);
   }
   if (!frames_dev || ((uintptr_t)frames_dev % 16)) return fail(p, SSOCT_EINVAL, "frames NULL or not 16-byte aligned");
@@ -138,8 +139,23 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   }
   p.noalloc_device = dev;
 
+  // The scratch ring starts where a workspace has its frame ring, which this
+  // path does not use, with as many slots as the array has room for before the
+  // intermediate (at least slots_noalloc, which noalloc_bytes counts).
+  const size_t slot_bytes = sizeof(float2) * (size_t)p.ny * p.wxp;
+  const size_t inter_bytes = sizeof(float2) * (size_t)p.wy * p.ntx * p.nl * kTile;
+  const int room = (int)std::min<size_t>((kNoAllocBytes - inter_bytes - p.off_ring) / slot_bytes, p.slots_alloc);
+  LateralSchedule sch = p.sch;
+  if (sch.slots > room) {
+    const LateralPick pick = lateral_pick(p.nl, sch.n_row + sch.n_col, room);
+    sch.lag = pick.lag;
+    sch.slots = pick.slots;
+  }
+  char* const scratch = ws + p.off_ring;
+  char* const inter = scratch + slot_bytes * room;  // a slot is a multiple of 512 bytes
+
   alignas(64) unsigned char tmap[128];
-  if (!encode_scratch_map_at(p, ws + p.off_scratch, tmap))
+  if (!encode_scratch_map_at(p, scratch, room, tmap))
     return fail(p, SSOCT_ECUDA, "cuTensorMapEncodeTiled failed for the no-allocation scratch ring");
 
   LateralParams lp;
@@ -155,12 +171,12 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   lp.cy = (const float2*)(ws + p.off_cy);
   lp.twx = (const float2*)(ws + p.off_twx);
   lp.twy = (const float2*)(ws + p.off_twy);
-  lp.scratch = (float2*)(ws + p.off_scratch);
-  lp.inter = (float2*)(ws + p.off_inter);
+  lp.scratch = (float2*)scratch;
+  lp.inter = (float2*)inter;
   lp.ctr = (Counters*)(ws + p.off_ctr);
   lp.rows_done = (unsigned*)(ws + p.off_ctr + sizeof(Counters));
   lp.cols_done = lp.rows_done + p.nl;
-  lp.sch = p.sch;
+  lp.sch = sch;
   lp.stage_rows = p.stage_rows;
   lp.stage_bytes = 0;
   lp.wait_ns = p.wait_ns;

@@ -138,6 +138,33 @@ struct LateralSchedule {
   }
 };
 
+// Default lag and ring slots of the lateral kernel for `frames` frames of
+// `items` work items each, with at most max_slots scratch slots.  A column item
+// waits for every row item of its frame and a row item for the column items of
+// the frame whose slot it reuses.  An item is published about 20 us after its
+// ticket was taken, and the 304 consumer groups of 152 SMs go through about
+// 1200 tickets in that time, so both distances (lag, and slots - lag) span 1200
+// items where the ring allows it; a frame count that fits the ring reuses no
+// slot.  Measured lateral times, paper order, against lags of 0.7 x 600 items
+// with four slots of slack: 256 x 256 x 512 353 -> 203 us, 512 x 512 x 256
+// 476 -> 347, 384 x 384 x 96 142 -> 94, 640 x 640 x 160 483 -> 401, 768 x 768 x
+// 200 722 -> 675, 1024 x 1024 x 256 1328 -> 1320; 2400 items gave no more.
+constexpr int kLateralItemsInFlight = 1200;
+struct LateralPick {
+  int lag, slots;
+};
+inline LateralPick lateral_pick(int frames, int items, int max_slots) {
+  const int depth = (kLateralItemsInFlight + items - 1) / items;
+  LateralPick r;
+  r.slots = 2 * depth < max_slots ? 2 * depth : max_slots;
+  r.lag = depth;
+  if (r.slots < frames && r.lag > r.slots / 2) r.lag = r.slots / 2;
+  if (r.slots > frames) r.slots = frames;
+  const int most = frames - (frames >= 4 ? 2 : 1);  // frames >= 1; lag < slots always
+  if (r.lag > most) r.lag = most;
+  return r;
+}
+
 // Everything the lateral kernel (rescale + chirp + row FFT, column FFT) reads.
 struct LateralParams {
   const uint16_t* frames;  // batch frame f at frames + ((ring_start + f) % nl) * nx * ny
@@ -224,6 +251,8 @@ struct Plan {
   int stage_rows;
   LateralSchedule sch;
   int slots_alloc = 0;       // scratch-ring slots the workspace holds (sch.slots <= slots_alloc)
+  int slots_noalloc = 0;     // ring slots counted in noalloc_bytes
+  size_t noalloc_bytes = 0;  // scratch the no-allocation path asks for (its size limit applies to this)
   bool use_tc = false;       // axial pass on the tensor cores (flag, or the autotuner's choice)
   // workspace layout (byte offsets)
   size_t off_ctr, off_xtab, off_ytab, off_cx, off_cy, off_cx2, off_cy2, off_ox, off_oy, off_twx, off_twy, off_twl;
@@ -330,10 +359,10 @@ size_t lateral_smem_bytes(const Plan& p);
 int lateral_col_band(int ny);
 
 // Used by the no-allocation entry point (noalloc.cu): the plan behind a handle,
-// a scratch-ring tensor map for scratch memory at an arbitrary device address,
+// a scratch-ring tensor map for `slots` slots at an arbitrary device address,
 // and a lateral launch that takes the tensor map and SM count explicitly.
 Plan& plan_of(ssoct_plan h);
-bool encode_scratch_map_at(const Plan& p, void* scratch_dev, void* map_out);
+bool encode_scratch_map_at(const Plan& p, void* scratch_dev, int slots, void* map_out);
 cudaError_t launch_lateral_with(const Plan& p, const LateralParams& lp, const void* tmap,
                                 int num_sms, cudaStream_t s);
 // The axial launch with the SM count given explicitly (the persistent streaming

@@ -127,33 +127,19 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// Tensor map over the scratch ring seen as float32 [slots * ny][2 * wxp]; one
-// box is a column band of the lateral kernel (2 * band floats x band_box_rows(ny) rows).
-bool encode_scratch_map(Plan& p) {
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const int band = lateral_col_band(p.ny);
-  cuuint64_t dims[2] = {(cuuint64_t)2 * p.wxp, (cuuint64_t)p.slots_alloc * p.ny};
-  cuuint64_t strides[1] = {(cuuint64_t)2 * p.wxp * sizeof(float)};
-  cuuint32_t box[2] = {(cuuint32_t)(2 * band), (cuuint32_t)band_box_rows(p.ny)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(reinterpret_cast<CUtensorMap*>(p.tmap), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p.ws + p.off_scratch,
-                   dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 }  // namespace
 
 namespace ssoct {
 
 Plan& plan_of(ssoct_plan h) { return h->p; }
 
-bool encode_scratch_map_at(const Plan& p, void* scratch_dev, void* map_out) {
+// Tensor map over a scratch ring seen as float32 [slots * ny][2 * wxp]; one
+// box is a column band of the lateral kernel (2 * band floats x band_box_rows(ny) rows).
+bool encode_scratch_map_at(const Plan& p, void* scratch_dev, int slots, void* map_out) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
   const int band = lateral_col_band(p.ny);
-  cuuint64_t dims[2] = {(cuuint64_t)2 * p.wxp, (cuuint64_t)p.slots_alloc * p.ny};
+  cuuint64_t dims[2] = {(cuuint64_t)2 * p.wxp, (cuuint64_t)slots * p.ny};
   cuuint64_t strides[1] = {(cuuint64_t)2 * p.wxp * sizeof(float)};
   cuuint32_t box[2] = {(cuuint32_t)(2 * band), (cuuint32_t)band_box_rows(p.ny)};
   cuuint32_t estr[2] = {1, 1};
@@ -337,35 +323,21 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.sch.nl = nlambda;
   p.sch.n_row = ny / p.rows_per_item;
   p.sch.n_col = (p.wx + p.cols_per_item - 1) / p.cols_per_item;
-  p.sch.lag = nlambda >= 3 ? 2 : nlambda - 1;
-  // a row item of frame f reuses the slot of frame f - slots, whose last column
-  // items were taken four steps earlier: enough slack that the wait is rare
-  p.sch.slots = p.sch.lag + 4;
-  // Slots the workspace holds (the autotuner may use them all).  A column item
-  // waits for every row item of its frame, so the lag has to span the frames
-  // whose items are in flight at once, about 600 on a 152-SM GPU (two groups
-  // computing and up to two buffers loaded per SM): 2.4 frames of 1024 x 1024,
-  // 9.5 of 512 x 512.  Smaller frames get more slots, as long as the ring
-  // stays within 64 MiB of L2.
+  // Ring slots the workspace holds (the autotuner may use them all): what the
+  // default schedule asks for, within 64 MiB of L2 (1024 x 1024: eight).
   {
-    const long long items = (long long)p.sch.n_row + p.sch.n_col;
-    const long long in_flight = (600 + items - 1) / items;
+    const int items = p.sch.n_row + p.sch.n_col;
     const long long slot_bytes = (long long)sizeof(float2) * ny * p.wxp;
-    long long n = std::max<long long>(p.sch.slots, in_flight + 4);
-    n = std::min<long long>(n, std::max<long long>(p.sch.slots, (64ll << 20) / slot_bytes));
-    n = std::min<long long>(n, std::max<long long>(p.sch.slots, nlambda));
-    p.slots_alloc = (int)n;
-    // default schedule: a lag of about 0.7 of the frames in flight (what the
-    // autotuner picked at 512 x 512 and 256 x 256; 3 at 1024 x 1024), four
-    // slots of slack
-    if (nlambda >= 3) {
-      const long long lag = std::min<long long>(std::max<long long>(2, (7 * in_flight + 9) / 10),
-                                                std::min<long long>(p.slots_alloc - 4, nlambda - 1));
-      if (lag >= 2) {
-        p.sch.lag = (int)lag;
-        p.sch.slots = (int)lag + 4;
-      }
-    }
+    const int in_l2 = (int)std::max<long long>(6, (64ll << 20) / slot_bytes);
+    // the ring that the no-allocation path's size limit is stated for
+    p.slots_noalloc = std::min({std::max(6, (600 + items - 1) / items + 4), in_l2, std::max(6, nlambda)});
+    // beyond 32 MiB the ring stays under a whole sweep's frame buffer (a short
+    // sweep of large frames would otherwise double its workspace)
+    const int most = std::max<long long>(6, std::min<long long>(in_l2, std::max<long long>(nlambda * 7 / 8, (32ll << 20) / slot_bytes)));
+    const LateralPick pick = lateral_pick(nlambda, items, most);
+    p.slots_alloc = std::max(pick.slots, p.slots_noalloc);
+    p.sch.lag = pick.lag;
+    p.sch.slots = pick.slots;
   }
   // input rows a row item stages: from the first row's base to the last row's base + 1
   int st = 0;
@@ -423,6 +395,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     p.off_red = take(sizeof(double) * kShRedDoubles);
   }
   p.ws_bytes = off;
+  p.noalloc_bytes = generic ? off : off - sizeof(float2) * (size_t)(p.slots_alloc - p.slots_noalloc) * ny * p.wxp;
   *out = h;
   return SSOCT_OK;
 }
@@ -498,7 +471,7 @@ ssoct_status ssoct_set_workspace(ssoct_plan h, void* dev_ptr, size_t bytes) {
       p.ws = nullptr;
       return cuda_fail(&p, e, "chirp table upload");
     }
-  } else if (!encode_scratch_map(p)) {
+  } else if (!encode_scratch_map_at(p, ws + p.off_scratch, p.slots_alloc, p.tmap)) {
     p.ws = nullptr;
     return fail(&p, SSOCT_ECUDA, "cuTensorMapEncodeTiled failed for the scratch ring");
   }
@@ -704,9 +677,10 @@ static ssoct_status sliding_update(Plan& p, cudaStream_t s, cudaEvent_t** ev_out
   if (k > 0) {
     const int slot0 = (int)(first % p.nl);
     LateralParams lp = lateral_params(p, (const uint16_t*)(p.ws + p.off_ring), slot0, slot0);
+    const LateralPick pick = lateral_pick(k, lp.sch.n_row + lp.sch.n_col, p.slots_alloc);
     lp.sch.nl = k;
-    lp.sch.lag = k >= 3 ? 2 : k - 1;
-    lp.sch.slots = lp.sch.lag + 4;  // never more than the plan's ring of scratch slots
+    lp.sch.lag = pick.lag;
+    lp.sch.slots = pick.slots;
     ssoct_status st = launch_lateral_pass(p, lp, s, &ev);
     if (st != SSOCT_OK) return st;
   }
