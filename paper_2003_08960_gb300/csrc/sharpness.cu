@@ -17,6 +17,7 @@
 // The DFTs here are the uncentred ones of the lateral kernel, with the centring
 // phase (-1)^n folded into c; the unit-modulus factors this moves onto V~ cancel
 // in W's round trip, so M is the same as with the centred transform.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <vector>
@@ -115,7 +116,8 @@ struct ShParams {
   float2* inter;           // [wy][ntx][nl][32] sweep-axis intermediate
   float2* qpart;           // [chunks][ny][nx] partial Q
   const float* vol;        // [nl][wy][wx] P_v
-  double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15
+  double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15, [19] float a1, a0, [20] block count
+  float sum_scale;         // power of two that keeps the squares of P_v in the float range
   int nx, ny, nl, x0, y0, wx, wy, ntx, tpc;
   int ring_start;          // frame t of the gate is frames[(ring_start + t) mod nl]
   float alpha2;            // |K|^2
@@ -182,19 +184,60 @@ __global__ void __launch_bounds__(kLatTW<NY> * Lat<NY>::N1) cols_fwd_kernel(cons
   });
 }
 
-// S1 = sum P, S2 = sum P^2 over the volume, FP64.
+// s + err = a + b exactly (Knuth 1969).
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+
+// S1 = sum P, S2 = sum P^2 over the volume, and from them the loss and the two
+// coefficients of dL/dP = a1 P + a0.  A pass over the volume should be bound by
+// its reads (20 us for 512 x 512 x 128); two FP64 operations and a conversion
+// per voxel at two FP64 operations per clock and SM took 240 (34 now, at six
+// blocks per SM; 41 at four, 47 at three, 41-44 at eight).  Each thread sums
+// in pairs of floats instead (two_sum; P^2 as its rounded square and the exact
+// remainder), which holds 48 bits, and the pairs meet in FP64.  P is scaled by a
+// power of two so that no square leaves the float range.
 __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constant__ ShParams p, size_t n) {
-  double s1 = 0.0, s2 = 0.0;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const double v = p.vol[i];
-    s1 += v;
-    s2 += v * v;
+  // two independent sums per thread: one alone waits for its own additions
+  float h1[2] = {0.f, 0.f}, l1[2] = {0.f, 0.f}, h2[2] = {0.f, 0.f}, l2[2] = {0.f, 0.f};
+  auto add = [&](int k, float v) {
+    float e;
+    v *= p.sum_scale;
+    h1[k] = two_sum(h1[k], v, e);
+    l1[k] += e;
+    const float q = __fmul_rn(v, v);
+    h2[k] = two_sum(h2[k], q, e);
+    l2[k] += e + fmaf(v, v, -q);
+  };
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  const float4* v4 = reinterpret_cast<const float4*>(p.vol);  // the volume is 16-byte aligned
+  const size_t n4 = n / 4;
+#pragma unroll 4
+  for (size_t i = first; i < n4; i += stride) {
+    const float4 v = __ldg(v4 + i);
+    add(0, v.x);
+    add(1, v.y);
+    add(0, v.z);
+    add(1, v.w);
   }
-  __shared__ double sh[2][kGradThreads / 32];
+  for (size_t i = n4 * 4 + first; i < n; i += stride) add(0, p.vol[i]);
+  // the lanes' pairs meet as pairs of floats, the warps' in FP64
+  auto join = [&](float& h, float& l, float h_o, float l_o) {
+    float e;
+    h = two_sum(h, h_o, e);
+    l += l_o + e;
+  };
+  join(h1[0], l1[0], h1[1], l1[1]);
+  join(h2[0], l2[0], h2[1], l2[1]);
   for (int o = 16; o; o >>= 1) {
-    s1 += __shfl_down_sync(0xffffffffu, s1, o);
-    s2 += __shfl_down_sync(0xffffffffu, s2, o);
+    join(h1[0], l1[0], __shfl_xor_sync(0xffffffffu, h1[0], o), __shfl_xor_sync(0xffffffffu, l1[0], o));
+    join(h2[0], l2[0], __shfl_xor_sync(0xffffffffu, h2[0], o), __shfl_xor_sync(0xffffffffu, l2[0], o));
   }
+  const double s1 = (double)h1[0] + l1[0], s2 = (double)h2[0] + l2[0];
+  __shared__ double sh[2][kGradThreads / 32];
   if (threadIdx.x % 32 == 0) {
     sh[0][threadIdx.x / 32] = s1;
     sh[1][threadIdx.x / 32] = s2;
@@ -206,8 +249,19 @@ __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constan
       a += sh[0][w];
       b += sh[1][w];
     }
-    atomicAdd(p.red + 0, a);
-    atomicAdd(p.red + 1, b);
+    const double inv = 1.0 / (double)p.sum_scale;  // a power of two: exact
+    atomicAdd(p.red + 0, a * inv);
+    atomicAdd(p.red + 1, b * inv * inv);
+    __threadfence();
+    // the last block to get here sees every sum
+    if (atomicAdd(reinterpret_cast<unsigned*>(p.red + 20), 1u) == gridDim.x - 1) {
+      __threadfence();
+      const double t1 = __ldcg(p.red + 0), t2 = __ldcg(p.red + 1);
+      float* c = reinterpret_cast<float*>(p.red + 19);
+      c[0] = (float)(-2.0 / (t1 * t1));
+      c[1] = (float)(2.0 * t2 / (t1 * t1 * t1));
+      p.red[2] = -t2 / (t1 * t1);
+    }
   }
 }
 
@@ -221,8 +275,9 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) axial_adj_kernel(const 
   float2* ex = reinterpret_cast<float2*>(smem);
   const int pix = threadIdx.x % kTile, j1 = threadIdx.x / kTile;
   float2* g = p.inter + ((size_t)blockIdx.y * p.ntx + blockIdx.x) * NL * kTile + pix;
-  const double s1 = p.red[0], s2 = p.red[1];
-  const float a1 = (float)(-2.0 / (s1 * s1)), a0 = (float)(2.0 * s2 / (s1 * s1 * s1));
+  // dL/dP = a1 P + a0, formed once by sums_kernel: the two FP64 divisions in
+  // every thread here took most of this kernel (115 us at 512 x 512 x 128)
+  const float a1 = reinterpret_cast<const float*>(p.red + 19)[0], a0 = reinterpret_cast<const float*>(p.red + 19)[1];
   float2 a[N2];
 #pragma unroll
   for (int j2 = 0; j2 < N2; ++j2) a[j2] = g[(j1 + N1 * j2) * kTile];
@@ -354,48 +409,123 @@ __host__ __device__ __forceinline__ void zernike15(double rho, double c1, double
   z[14] = q10 * r4 * s4;
 }
 
+// The same polynomials in the monomials X^a Y^b, a + b <= 4 (X = rho cos, Y =
+// rho sin), in the order of mono_a / mono_b: Z_j = sum_i kZernike[j][i] X^a Y^b.
+#define SSOCT_ZERNIKE_ROWS \
+  {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {0, 2, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {0, 0, 2, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {-R3, 0, 0, 2 * R3, 0, 2 * R3, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {0, 0, 0, 0, 2 * R6, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {0, 0, 0, R6, 0, -R6, 0, 0, 0, 0, 0, 0, 0, 0, 0}, \
+  {0, 0, -2 * R8, 0, 0, 0, 0, 3 * R8, 0, 3 * R8, 0, 0, 0, 0, 0}, \
+  {0, -2 * R8, 0, 0, 0, 0, 3 * R8, 0, 3 * R8, 0, 0, 0, 0, 0, 0}, \
+  {0, 0, 0, 0, 0, 0, 0, 3 * R8, 0, -R8, 0, 0, 0, 0, 0}, \
+  {0, 0, 0, 0, 0, 0, R8, 0, -3 * R8, 0, 0, 0, 0, 0, 0}, \
+  {R5, 0, 0, -6 * R5, 0, -6 * R5, 0, 0, 0, 0, 6 * R5, 0, 12 * R5, 0, 6 * R5}, \
+  {0, 0, 0, -3 * R10, 0, 3 * R10, 0, 0, 0, 0, 4 * R10, 0, 0, 0, -4 * R10}, \
+  {0, 0, 0, 0, -6 * R10, 0, 0, 0, 0, 0, 0, 8 * R10, 0, 8 * R10, 0}, \
+  {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, R10, 0, -6 * R10, 0, R10}, \
+  {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 4 * R10, 0, -4 * R10, 0}
+constexpr double R3 = 1.7320508075688772935, R5 = 2.2360679774997896964, R6 = 2.4494897427831780982,
+                 R8 = 2.8284271247461900976, R10 = 3.1622776601683793320;
+constexpr int kMono = 15;
+static __constant__ double kZernikeDev[15][kMono] = {SSOCT_ZERNIKE_ROWS};
+static const double kZernike[15][kMono] = {SSOCT_ZERNIKE_ROWS};
+#undef SSOCT_ZERNIKE_ROWS
+__host__ __device__ constexpr int mono_a(int i) {  // power of X: 1, X Y, X2 XY Y2, X3 X2Y XY2 Y3, ...
+  return i == 0 ? 0 : i < 3 ? 2 - i : i < 6 ? 5 - i : i < 10 ? 9 - i : 14 - i;
+}
+__host__ __device__ constexpr int mono_b(int i) {
+  return i == 0 ? 0 : i < 3 ? i - 1 : i < 6 ? i - 3 : i < 10 ? i - 6 : i - 10;
+}
+
 namespace {
 
+// Threads of a block along x in grad_kernel and pupil_table_kernel (nx is a
+// multiple of 64).
+__host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 : nx % 128 == 0 ? 128 : 64; }
+
+// dL/dz and dL/dc_j: sums over the sensor of M r^2 and M Z_j, M = -Im(c P Q).
+// All of them are combinations of the 15 moments sum M X^a Y^b, so a pixel costs
+// the moments along y only (five FP64 fused steps); a thread keeps its column x,
+// and X^a and the Zernike combinations come in once per thread and per block.
+// The chunks of Q are added as pairs of floats (two_sum).  Evaluating the
+// polynomials and adding the chunks in FP64 per pixel (two FP64 operations per
+// clock and SM) took 98 us at 512 x 512 x 128; 31 us now (three blocks per SM; 36
+// with two, 33 with four: each thread still ends with some 35 FP64 operations).
+// The reads of Q alone would take 6.
 __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks) {
-  double acc[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) acc[j] = 0.0;
+  const int tx = grid_tx(p.nx), ry = kGradThreads / tx;
+  const int x = blockIdx.x * tx + threadIdx.x % tx;
   const size_t npix = (size_t)p.nx * p.ny;
-  const double cxp = p.nx / 2.0, cyp = p.ny / 2.0;
   const double inv_radius = 2.0 / (double)min(p.nx, p.ny);  // rho = r_pix / (min(nx, ny) / 2)
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < npix; i += (size_t)gridDim.x * blockDim.x) {
-    double qx = 0.0, qy = 0.0;
+  double my[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // sum_y M Y^b of this column
+  for (int y = blockIdx.y * ry + threadIdx.x / tx; y < p.ny; y += gridDim.y * ry) {
+    const size_t i = (size_t)y * p.nx + x;
+    float qx = 0.f, lx = 0.f, qy = 0.f, ly = 0.f;
+#pragma unroll 16
     for (int c = 0; c < chunks; ++c) {
-      const float2 q = p.qpart[(size_t)c * npix + i];
-      qx += q.x;
-      qy += q.y;
+      const float2 q = __ldg(p.qpart + (size_t)c * npix + i);
+      float e;
+      qx = two_sum(qx, q.x, e);
+      lx += e;
+      qy = two_sum(qy, q.y, e);
+      ly += e;
     }
-    const float2 cp = p.cp[i];
-    const double m = -((double)cp.x * qy + (double)cp.y * qx);  // -Im(c P Q)
-    const double dx = (double)(i % p.nx) - cxp, dy = (double)(i / p.nx) - cyp;
-    const double r2 = dx * dx + dy * dy;
-    const double rp = sqrt(r2);
-    const double c1 = rp > 0.0 ? dx / rp : 1.0, s1 = rp > 0.0 ? dy / rp : 0.0;
-    double z[15];
-    zernike15(rp * inv_radius, c1, s1, z);
-    acc[0] += r2 * m;
-#pragma unroll
-    for (int j = 0; j < 15; ++j) acc[1 + j] += z[j] * m;
+    // M = -Im(c P Q), the products and their sum as pairs of floats too
+    const float2 cp = __ldg(p.cp + i);
+    const float u = __fmul_rn(cp.x, qy), v = __fmul_rn(cp.y, qx);
+    float e;
+    const float h = two_sum(u, v, e);
+    e += fmaf(cp.x, qy, -u) + fmaf(cp.y, qx, -v) + fmaf(cp.x, ly, cp.y * lx);
+    const double m = -((double)h + (double)e);
+    const double yy = (double)(y - p.ny / 2) * inv_radius, y2 = yy * yy;
+    my[0] += m;
+    my[1] = fma(m, yy, my[1]);
+    my[2] = fma(m, y2, my[2]);
+    my[3] = fma(m, y2 * yy, my[3]);
+    my[4] = fma(m, y2 * y2, my[4]);
   }
-  __shared__ double sh[16][kGradThreads / 32];
+  const double xx = (double)(x - p.nx / 2) * inv_radius;
+  const double xp[5] = {1.0, xx, xx * xx, xx * xx * xx, (xx * xx) * (xx * xx)};
+  double mom[16];
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    double v = acc[j];
-    for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x % 32 == 0) sh[j][threadIdx.x / 32] = v;
+  for (int i = 0; i < kMono; ++i) mom[i] = mono_a(i) ? my[mono_b(i)] * xp[mono_a(i)] : my[mono_b(i)];
+  mom[15] = 0.0;
+  // warp sum of the 16 values: each step halves the values a lane holds
+  const int lane = threadIdx.x % 32;
+#pragma unroll
+  for (int h = 8; h; h >>= 1) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double keep = up ? mom[i + h] : mom[i], send = up ? mom[i] : mom[i + h];
+      mom[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+    }
+  }
+  // lane l now holds value l % 16, summed over the lanes of its half warp
+  double v = mom[0];
+  v += __shfl_xor_sync(0xffffffffu, v, 16);
+  __shared__ double sh[16][kGradThreads / 32];
+  __shared__ double tot[16];
+  if (lane < 16) sh[lane][threadIdx.x / 32] = v;
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    double t = 0.0;
+    for (int w = 0; w < kGradThreads / 32; ++w) t += sh[threadIdx.x][w];
+    tot[threadIdx.x] = t;
   }
   __syncthreads();
   if (threadIdx.x < 16) {
-    double v = 0.0;
-    for (int w = 0; w < kGradThreads / 32; ++w) v += sh[threadIdx.x][w];
-    atomicAdd(p.red + 3 + threadIdx.x, threadIdx.x == 0 ? v * p.scale_z : v);
+    double t = 0.0;
+    if (threadIdx.x == 0) {
+      t = (tot[3] + tot[5]) / (inv_radius * inv_radius) * p.scale_z;  // sum M r_pix^2
+    } else {
+      for (int i = 0; i < kMono; ++i) t += kZernikeDev[threadIdx.x - 1][i] * tot[i];
+    }
+    atomicAdd(p.red + 3 + threadIdx.x, t);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) p.red[2] = -p.red[1] / (p.red[0] * p.red[0]);
 }
 
 // ----------------------------------------------------------------- launchers
@@ -507,43 +637,81 @@ namespace {
 
 struct PupilParams {
   float2* cp;
-  int nx, ny, ncoeffs;
-  double alpha;
-  double c[15];
+  const float4* cis;  // [256] exp(i pi k / 128) as pairs of floats (re hi, re lo, im hi, im lo)
+  int nx, ny;
+  double c[kMono];    // phase / pi as a polynomial in the pixel offsets from the centre
 };
 
-// c P per sensor pixel, the device twin of build_pupil_table: phases reduced in
-// units of pi in float64, one rounding to float32 at the end.
+constexpr int kPupilRows = 8;  // rows of a block: their polynomials in x come from the first threads
+
+// c P per sensor pixel, the device twin of build_pupil_table.  The phase over pi
+// (chirp and Zernike sum, a polynomial of degree four) is evaluated and reduced
+// in float64, split into the nearest 1/128 and a remainder, and the remainder
+// turns the tabulated exponential (held to 48 bits) by its series: one rounding
+// to float32 at the end, as with the float64 sine and cosine, square root and
+// fmod per pixel that took 78 us at 512 x 512 (two FP64 operations per clock and
+// SM: about 15 per pixel now, 9 us).
 __global__ void __launch_bounds__(256) pupil_table_kernel(const __grid_constant__ PupilParams p) {
-  const size_t npix = (size_t)p.nx * p.ny;
-  const double inv_radius = 2.0 / (double)min(p.nx, p.ny);
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < npix; i += (size_t)gridDim.x * blockDim.x) {
-    const int n = (int)(i % p.nx), l = (int)(i / p.nx);
-    const double dx = n - p.nx / 2.0, dy = l - p.ny / 2.0;
-    double turns = -(fmod(p.alpha * dx * dx, 2.0) + (double)(n & 1)) - (fmod(p.alpha * dy * dy, 2.0) + (double)(l & 1));
-    const double rp = sqrt(dx * dx + dy * dy);
-    double z[15];
-    zernike15(rp * inv_radius, rp > 0.0 ? dx / rp : 1.0, rp > 0.0 ? dy / rp : 0.0, z);
-    double phi = 0.0;
-    for (int j = 0; j < p.ncoeffs; ++j) phi += p.c[j] * z[j];
-    turns += fmod(phi / 3.14159265358979323846, 2.0);
-    double sn, cs;
-    sincospi(turns, &sn, &cs);
-    p.cp[i] = make_float2((float)cs, (float)sn);
+  __shared__ double row[kPupilRows][5];
+  __shared__ float4 cis[256];
+  const int y0 = blockIdx.y * kPupilRows;
+  cis[threadIdx.x] = __ldg(p.cis + threadIdx.x);
+  if (threadIdx.x < kPupilRows * 5) {
+    const int r = threadIdx.x / 5, a = threadIdx.x % 5;
+    const double dy = (double)(y0 + r - p.ny / 2);
+    double v = 0.0;  // sum over b of c[a, b] dy^b
+    for (int i = kMono - 1; i >= 0; --i)
+      if (mono_a(i) == a) v = v * dy + p.c[i];
+    row[r][a] = v;
+  }
+  __syncthreads();
+  const int tx = grid_tx(p.nx);
+  const int x = blockIdx.x * tx + threadIdx.x % tx;
+  const double dx = (double)(x - p.nx / 2);
+  for (int r = threadIdx.x / tx; r < kPupilRows && y0 + r < p.ny; r += 256 / tx) {
+    const double* k = row[r];
+    const double t = (((k[4] * dx + k[3]) * dx + k[2]) * dx + k[1]) * dx + k[0];
+    const double m = rint(t * 128.0);             // nearest 1/128
+    const float d = (float)(t - m * (1.0 / 128.0)) * 3.14159265f;
+    // m mod 256 selects the table entry (period 2), and the centring phase (-1)^(n + l) adds a half turn
+    const int e = ((int)(long long)m + 128 * ((x + y0 + r) & 1)) & 255;
+    const float4 w = cis[e];
+    const float d2 = d * d;
+    const float s = fmaf(d2 * d, -1.f / 6.f, d);
+    const float c1 = d2 * fmaf(d2, 1.f / 24.f, -0.5f);  // cos d - 1
+    const float re = w.x + (w.y + fmaf(w.x, c1, -w.z * s));
+    const float im = w.z + (w.w + fmaf(w.z, c1, w.x * s));
+    p.cp[(size_t)(y0 + r) * p.nx + x] = make_float2(re, im);
   }
 }
 
 }  // namespace
 
+void pupil_cis_table(std::vector<float4>& out) {
+  out.resize(256);
+  for (int k = 0; k < 256; ++k) {
+    const double a = 3.14159265358979323846 * k / 128.0, c = std::cos(a), s = std::sin(a);
+    const float ch = (float)c, sh = (float)s;
+    out[k] = make_float4(ch, (float)(c - ch), sh, (float)(s - sh));
+  }
+}
+
 cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s) {
   PupilParams p;
   p.cp = (float2*)(pl.ws + pl.off_cp);
+  p.cis = (const float4*)(pl.ws + pl.off_cis);
   p.nx = pl.nx;
   p.ny = pl.ny;
-  p.ncoeffs = pl.sh_ncoeffs;
-  p.alpha = pl.sh_alpha;
-  for (int j = 0; j < 15; ++j) p.c[j] = j < pl.sh_ncoeffs ? pl.sh_coeffs[j] : 0.0;
-  pupil_table_kernel<<<2 * pl.num_sms, 256, 0, s>>>(p);
+  const double pi = 3.14159265358979323846, inv_radius = 2.0 / (double)(pl.nx < pl.ny ? pl.nx : pl.ny);
+  for (int i = 0; i < kMono; ++i) {
+    double v = 0.0;
+    for (int j = 0; j < pl.sh_ncoeffs; ++j) v += pl.sh_coeffs[j] * kZernike[j][i];
+    p.c[i] = v / pi * std::pow(inv_radius, mono_a(i) + mono_b(i));
+  }
+  p.c[3] -= pl.sh_alpha;  // the input chirp, -alpha (dx^2 + dy^2)
+  p.c[5] -= pl.sh_alpha;
+  const int tx = grid_tx(pl.nx);
+  pupil_table_kernel<<<dim3(pl.nx / tx, (pl.ny + kPupilRows - 1) / kPupilRows), 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -596,6 +764,14 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   p.tpc = pl.sh_tpc;
   p.alpha2 = (float)(pl.sh_alpha * pl.sh_alpha);
   p.scale_z = 3.14159265358979323846 * pl.sh_alpha / pl.sh_z;
+  {
+    // sum P <= |K|^2 (65535 nx ny nl)^2 (Parseval), which the scale takes to 2^62:
+    // the sum of squares stays under 2^124, and P down to 1e-36 of it counts in full
+    int ex = 0;
+    const double top = 65535.0 * pl.nx * pl.ny * pl.nl * pl.sh_alpha;
+    std::frexp(top * top, &ex);
+    p.sum_scale = (float)std::ldexp(1.0, std::max(-126, std::min(126, 62 - ex)));
+  }
   const int chunks = (pl.nl + pl.sh_tpc - 1) / pl.sh_tpc;
 
   cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
@@ -617,14 +793,16 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   }
   const size_t nvox = (size_t)pl.nl * pl.wy * pl.wx;
   if (e == cudaSuccess) {
-    sums_kernel<<<2 * pl.num_sms, kGradThreads, 0, s>>>(p, nvox);
+    sums_kernel<<<6 * pl.num_sms, kGradThreads, 0, s>>>(p, nvox);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = axial_adj_any(p, s);
   if (e == cudaSuccess) e = cols_any(true, p, s);
   if (e == cudaSuccess) e = rows_any(true, p, chunks, s);
   if (e == cudaSuccess) {
-    grad_kernel<<<2 * pl.num_sms, kGradThreads, 0, s>>>(p, chunks);
+    const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;
+    const int gy = std::min((p.ny + ry - 1) / ry, std::max(1, 3 * pl.num_sms / gx));
+    grad_kernel<<<dim3(gx, gy), kGradThreads, 0, s>>>(p, chunks);
     e = cudaGetLastError();
   }
   return e;

@@ -258,7 +258,7 @@ struct Plan {
   size_t off_ctr, off_xtab, off_ytab, off_cx, off_cy, off_cx2, off_cy2, off_ox, off_oy, off_twx, off_twy, off_twl;
   size_t off_twra = 0;       // twiddles of the tiled first pass's split (ra_split_n1)
   size_t off_tcb, off_wq, off_ring, off_scratch, off_inter, ws_bytes;
-  size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0;  // SSOCT_FLAG_PUPIL regions
+  size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0, off_cis = 0;  // SSOCT_FLAG_PUPIL regions
   // Frame sizes the persistent lateral kernel does not compile (384, 640, 768)
   // take the two-pass lateral path of sharpness.cu: chirp table and frame buffer.
   bool generic = false;
@@ -343,14 +343,17 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
                             int num_sms, cudaStream_t s);
 // Aberration path (sharpness.cu): sizes it compiles, the c P table, and the
 // forward + adjoint launches that leave loss and gradient in the FP64 block at
-// off_red ([0] S1, [1] S2, [2] loss, [3] dL/dz, [4..18] dL/dc_1..15).
-constexpr int kShRedDoubles = 19;
+// off_red ([0] S1, [1] S2, [2] loss, [3] dL/dz, [4..18] dL/dc_1..15, then the
+// two coefficients of dL/dP and a block count of the kernels).
+constexpr int kShRedDoubles = 21;
 bool sharpness_supported(int nx, int ny, int nl);
 bool generic_lateral_supported(int nx, int ny);
 // Eq. 5 + Eq. 6 as a row pass and a column pass through the frame buffer at
 // off_F, for frames[(ring_start + t) mod nl]; writes the sweep-axis intermediate.
 cudaError_t launch_lateral_generic(const Plan& pl, const uint16_t* frames, int ring_start, cudaStream_t s);
 void build_pupil_table(int nx, int ny, double alpha, const double* coeffs, int ncoeffs, std::vector<float2>& out);
+// exp(i pi k / 128), k = 0 .. 255, as pairs of floats (re hi, re lo, im hi, im lo).
+void pupil_cis_table(std::vector<float4>& out);
 cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, cudaStream_t s);
 cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s);
 // Dynamic shared memory of the lateral kernel for a plan (bytes).

@@ -393,6 +393,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     p.off_cp = take(sizeof(float2) * (size_t)nx * ny);
     p.off_Q = take(sizeof(float2) * chunks * ny * nx);
     p.off_red = take(sizeof(double) * kShRedDoubles);
+    p.off_cis = take(sizeof(float4) * 256);
   }
   p.ws_bytes = off;
   p.noalloc_bytes = generic ? off : off - sizeof(float2) * (size_t)(p.slots_alloc - p.slots_noalloc) * ny * p.wxp;
@@ -463,6 +464,15 @@ ssoct_status ssoct_set_workspace(ssoct_plan h, void* dev_ptr, size_t bytes) {
   p.ws = ws;
   p.stream_count = 0;
   p.lat_upto = -1;
+  if (p.flags & SSOCT_FLAG_PUPIL) {
+    std::vector<float4> cis;
+    pupil_cis_table(cis);
+    e = cudaMemcpy(ws + p.off_cis, cis.data(), sizeof(float4) * cis.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      p.ws = nullptr;
+      return cuda_fail(&p, e, "pupil table upload");
+    }
+  }
   if (p.generic) {
     std::vector<float2> cg;
     build_pupil_table(p.nx, p.ny, p.alpha, nullptr, 0, cg);  // the input chirp alone
