@@ -8,9 +8,11 @@
 // complex values (contiguous in the intermediate) go through the
 // N_lambda-point DFT as N2-point DFTs in registers, a twiddle, an exchange
 // through shared memory and N1-point DFTs, and leave as 128-byte runs of the
-// volume per depth bin.  Sweeps of 64 to 256 frames take the persistent
-// streaming form (axial_stream_kernel: TMA-fed ring of stage buffers, two
-// consumer groups per SM); the others one CTA per tile (axial_kernel).
+// volume per depth bin.  Sweeps of 64 frames and more take the persistent
+// streaming form (axial_stream_kernel: TMA-fed ring of stage buffers, two or
+// more consumer groups per SM); those of 16 and 32 one CTA per tile (axial_kernel).
+#include <algorithm>
+
 #include <cuda.h>
 
 #include "fft_common.cuh"
@@ -67,29 +69,40 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) axial_kernel(const __gr
   });
 }
 
-// Streaming form for sweeps of up to 256 frames: one persistent CTA per SM,
-// two consumer groups and a ring of shared-memory stage buffers.  Whole tiles
-// (N_lambda x 32 complex values, contiguous in the intermediate) arrive by 1D
-// TMA bulk copies, a ring's worth ahead; group g computes the CTA's tiles
-// g, g + 2, ... with the same two-stage DFT as axial_kernel, doing the exchange
-// in place in the stage buffer, and once all its threads are done with a
-// buffer one of them issues the copy of the tile kStages further on into it.
-// The loads never wait for the arithmetic, so HBM keeps streaming.
-constexpr int kAxGroups = 2;
+// Streaming form for sweeps of 64 frames and more: one persistent CTA per SM,
+// consumer groups and a ring of shared-memory stage buffers.  Units of kPix
+// pixels (N_lambda x kPix complex values: a whole tile, contiguous in the
+// intermediate, by one 1D TMA bulk copy; half a tile for 512 frames, whose
+// tiles would fill the ring alone, by 2D tensor copies of 256 frames) arrive a
+// ring's worth ahead; group g computes the CTA's units g, g + kGroups, ... with
+// the same two-stage DFT as axial_kernel, doing the exchange in place in the
+// stage buffer, and once all its threads are done with a buffer one of them
+// issues the copy of the unit kStages further on into it.  The loads never wait
+// for the arithmetic, so HBM keeps streaming.
 constexpr size_t kAxRingBytes = 192 * 1024;
 constexpr unsigned long long kAxWaitNs = 4000000000ull;  // 4 s
 
+constexpr int lcm_of(int a, int b) {
+  int m = a;
+  while (m % b != 0) m += a;
+  return m;
+}
+
 template <int NL>
 struct AxStream {
-  static constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
-  static constexpr int kGroupThreads = kTile * N1;
-  static constexpr int kThreadsAll = kAxGroups * kGroupThreads;
-  static constexpr size_t kTileBytes = (size_t)NL * kTile * sizeof(float2);
-  static constexpr int kStages = kAxRingBytes / kTileBytes > 8 ? 8 : (int)(kAxRingBytes / kTileBytes);
-  // one full barrier per tile index mod lcm(kStages, kAxGroups): each is waited
+  static constexpr int N1 = ax_split_n1(NL), N2 = NL / N1;
+  using S2 = Stage2<NL, N1>;
+  static constexpr int kPix = NL > 256 ? kTile / 2 : kTile;
+  static constexpr int kUnits = kTile / kPix;  // per tile
+  static constexpr int kGroups = NL == 96 ? 4 : NL == 160 ? 3 : 2;
+  static constexpr int kGroupThreads = kPix * N1;
+  static constexpr int kThreadsAll = kGroups * kGroupThreads;
+  static constexpr size_t kUnitBytes = (size_t)NL * kPix * sizeof(float2);
+  static constexpr int kStages = kAxRingBytes / kUnitBytes > 8 ? 8 : (int)(kAxRingBytes / kUnitBytes);
+  // one full barrier per unit index mod lcm(kStages, kGroups): each is waited
   // on by one group only, which has consumed its previous fill, and its fills
   // follow one another through the buffer chain t -> t + kStages
-  static constexpr int kFull = kStages % kAxGroups == 0 ? kStages : kStages * kAxGroups;
+  static constexpr int kFull = lcm_of(kStages, kGroups);
 };
 
 __device__ bool mbar_wait_bounded(uint64_t* b, unsigned parity, unsigned long long limit_ns) {
@@ -115,18 +128,28 @@ __device__ __forceinline__ void group_sync(int id) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(T) : "memory");
 }
 
-// Copy of the CTA's tile t (global tile blockIdx.x + t * gridDim.x) into stage
+// Copy of the CTA's unit t (global unit blockIdx.x + t * gridDim.x) into stage
 // buffer t mod kStages; fills[] counts the copies issued on each full barrier.
 template <int NL>
-__device__ __forceinline__ void axial_fill(const AxialParams& p, unsigned char* ring, uint64_t* full_bar,
-                                           unsigned* fills, int t) {
+__device__ __forceinline__ void axial_fill(const AxialParams& p, const CUtensorMap* imap, unsigned char* ring,
+                                           uint64_t* full_bar, unsigned* fills, int t) {
   using S = AxStream<NL>;
   const int f = t % S::kFull;
   atomicAdd(&fills[f], 1u);
-  mbar_arrive_tx(&full_bar[f], (unsigned)S::kTileBytes);
-  const size_t gt = blockIdx.x + (size_t)t * gridDim.x;
-  tma_load_1d(ring + (size_t)(t % S::kStages) * S::kTileBytes, p.inter + gt * NL * kTile, (unsigned)S::kTileBytes,
-              &full_bar[f]);
+  mbar_arrive_tx(&full_bar[f], (unsigned)S::kUnitBytes);
+  const size_t gu = blockIdx.x + (size_t)t * gridDim.x;
+  unsigned char* dst = ring + (size_t)(t % S::kStages) * S::kUnitBytes;
+  if constexpr (S::kUnits == 1) {
+    tma_load_1d(dst, p.inter + gu * NL * kTile, (unsigned)S::kUnitBytes, &full_bar[f]);
+  } else {
+    // boxes of 256 frames: the destinations are multiples of 256 x kPix x 8
+    // bytes, the x start a multiple of 128 bytes
+    static_assert(NL % 256 == 0 && (256 * S::kPix * sizeof(float2)) % 128 == 0, "whole, aligned tensor copies");
+#pragma unroll
+    for (int r = 0; r < NL / 256; ++r)
+      tma_load_2d(dst + (size_t)r * 256 * S::kPix * sizeof(float2), imap, (int)(gu % S::kUnits) * 2 * S::kPix,
+                  (int)(gu / S::kUnits) * NL + r * 256, &full_bar[f]);
+  }
 }
 
 // End of a streaming tile: the depth bins q = k2 + N2 k1 this thread holds (a[])
@@ -134,14 +157,16 @@ __device__ __forceinline__ void axial_fill(const AxialParams& p, unsigned char* 
 // if CPLX, V with the output chirp and K into the complex volume.
 template <int NL, bool MAG, bool CPLX>
 __device__ __forceinline__ void axial_epilogue(const AxialParams& p, const float2* a, int j1, int kyw, int kxw) {
-  constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
+  using S2 = typename AxStream<NL>::S2;
+  constexpr int N1 = S2::N1, N2 = S2::N2;
   const size_t plane = (size_t)p.wy * p.wx;
   float* vol = p.vol + (size_t)kyw * p.wx + kxw;
   float2 of = make_float2(0.f, 0.f);
   if constexpr (CPLX) of = cmul(ldg2(p.ox + kxw), ldg2(p.oy + kyw));
-  static_for<0, N2 / N1>([&](auto I) {
+  static_for<0, S2::NI>([&](auto I) {
     constexpr int ii = decltype(I)::value;
     const int k2 = j1 + N1 * ii;
+    if (!S2::live(ii, j1)) return;
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) {
       const int q = k2 + N2 * k1;
@@ -156,16 +181,18 @@ __device__ __forceinline__ void axial_epilogue(const AxialParams& p, const float
 
 template <int NL>
 __global__ void __launch_bounds__(AxStream<NL>::kThreadsAll, 1)
-    axial_stream_kernel(const __grid_constant__ AxialParams p) {
+    axial_stream_kernel(const __grid_constant__ AxialParams p, const __grid_constant__ CUtensorMap imap) {
   using S = AxStream<NL>;
-  constexpr int N1 = S::N1, N2 = S::N2, T = S::kGroupThreads;
-  static_assert(N2 % N1 == 0, "the second stage needs N1 | N2");
-  extern __shared__ __align__(16) unsigned char smem[];  // 16 B: the bulk copies need no more
+  using S2 = typename S::S2;
+  constexpr int N1 = S::N1, N2 = S::N2, T = S::kGroupThreads, P = S::kPix;
+  static_assert(S::kThreadsAll <= 1024 && T % 32 == 0, "whole warps, one CTA");
+  extern __shared__ __align__(1024) unsigned char smem_ax[];  // tensor copies need 128
+  unsigned char* smem = smem_ax;
   __shared__ __align__(8) uint64_t full_bar[S::kFull];
   __shared__ unsigned fills[S::kFull];
   const int tid = threadIdx.x;
-  const int ntiles = p.ntx * p.wy;
-  const int mine = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int nunits = p.ntx * p.wy * S::kUnits;
+  const int mine = (int)blockIdx.x < nunits ? (nunits - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   if (tid == 0) {
 #pragma unroll
     for (int b = 0; b < S::kFull; ++b) {
@@ -173,16 +200,17 @@ __global__ void __launch_bounds__(AxStream<NL>::kThreadsAll, 1)
       fills[b] = 0u;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int t = 0; t < S::kStages && t < mine; ++t) axial_fill<NL>(p, smem, full_bar, fills, t);
+    for (int t = 0; t < S::kStages && t < mine; ++t) axial_fill<NL>(p, &imap, smem, full_bar, fills, t);
   }
   __syncthreads();
   const int g = tid / T;
   const int lt = tid % T;
-  const int pix = lt % kTile;
-  const int j1 = lt / kTile;
-  for (int i = g, prev = -1;; prev = i, i += kAxGroups) {
+  const int pix = lt % P;
+  const int j1 = lt / P;
+  for (int i = g, prev = -1;; prev = i, i += S::kGroups) {
     group_sync<T>(1 + g);  // every thread of the group is done with tile prev's buffer
-    if (lt == 0 && prev >= 0 && prev + S::kStages < mine) axial_fill<NL>(p, smem, full_bar, fills, prev + S::kStages);
+    if (lt == 0 && prev >= 0 && prev + S::kStages < mine)
+      axial_fill<NL>(p, &imap, smem, full_bar, fills, prev + S::kStages);
     if (i >= mine) break;
     // one thread waits for the tile; the others sleep at the group barrier
     bool ok = true;
@@ -191,29 +219,31 @@ __global__ void __launch_bounds__(AxStream<NL>::kThreadsAll, 1)
       if (!ok) atomicOr(p.err, kErrAxial);
     }
     if (group_sync_or<T>(1 + g, !ok)) break;
-    float2* ex = reinterpret_cast<float2*>(smem + (size_t)(i % S::kStages) * S::kTileBytes);
-    float2 a[N2];
+    float2* ex = reinterpret_cast<float2*>(smem + (size_t)(i % S::kStages) * S::kUnitBytes);
+    float2 a[S2::A];
 #pragma unroll
-    for (int j2 = 0; j2 < N2; ++j2) a[j2] = ex[(j1 + N1 * j2) * kTile + pix];
+    for (int j2 = 0; j2 < N2; ++j2) a[j2] = ex[(j1 + N1 * j2) * P + pix];
     Dft<N2, -1>::template run<1, 0>(a);
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) a[k2] = cmul(a[k2], ldg2(p.twl + k2 * N1 + j1));
     // t = k2 N1 + j1 runs over the same frames j1 + N1 j2 this thread read
 #pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * kTile + pix] = a[k2];
+    for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * P + pix] = a[k2];
     // these writes come before the buffer's next TMA fill (async proxy)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     group_sync<T>(1 + g);
-    static_for<0, N2 / N1>([&](auto I) {
+    static_for<0, S2::NI>([&](auto I) {
       constexpr int ii = decltype(I)::value;
       const int k2 = j1 + N1 * ii;
+      if (!S2::live(ii, j1)) return;
 #pragma unroll
-      for (int jj = 0; jj < N1; ++jj) a[ii * N1 + jj] = ex[(k2 * N1 + jj) * kTile + pix];
+      for (int jj = 0; jj < N1; ++jj) a[ii * N1 + jj] = ex[(k2 * N1 + jj) * P + pix];
       Dft<N1, -1>::template run<1, ii * N1>(a);
     });
-    const int gt = (int)blockIdx.x + i * (int)gridDim.x;
-    const int kyw = gt / p.ntx;
-    const int kxw = (gt - kyw * p.ntx) * kTile + pix;
+    const int gu = (int)blockIdx.x + i * (int)gridDim.x;
+    const int row = p.ntx * S::kUnits;
+    const int kyw = gu / row;
+    const int kxw = (gu - kyw * row) * P + pix;
     if (kxw >= p.wx) continue;
     // the options are tested once per tile: inside the unrolled loop they were
     // predicated on every value
@@ -343,13 +373,6 @@ struct RescaleAxialTileParams {
 };
 
 constexpr int kRaStrip = 64;  // pixels per tile (two per complex series)
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-          "r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
 
 // Eq. 5 at strip pixel k of a frame whose two staged source rows are r0, r1.
 __device__ __forceinline__ float ra_sample(int k, const StripTap& xs, const Tap& yt, const uint16_t* r0,
@@ -531,7 +554,7 @@ __global__ void __launch_bounds__(RaTile<NL>::kThreads, 1)
 struct GateCutsParams {
   const float2* inter;   // [wy][ntx][nl][32]
   const float2* wq;      // [nl] exp(-2 pi i k / nl)
-  const float2* twl;     // [N2l][N1l], sign - (the axial kernel's table)
+  const float2* twl;     // [N2][N1] of ax_split_n1, sign - (the axial kernel's table)
   float* xy;             // [wy][wx] or NULL
   float* xz;             // [nl][wx] or NULL
   float* yz;             // [nl][wy] or NULL
@@ -591,69 +614,105 @@ struct XySlideParams {
 // slot t changes it by (h_new - h_old) exp(-2 pi i z0 t / nl): one pass with
 // sign -1 over the slots about to be overwritten (before the lateral pass) and
 // one with sign +1 after it read k slots per pixel instead of nl.
+//
+// Bound by the reads of the slots (109 MB for 13 frames of 1024 x 1024): a
+// thread takes two adjacent pixels, so that a load is 16 bytes, and keeps
+// kSlideAhead slots in flight.  One pixel a thread and one slot at a time took
+// 38 us there (3.2 TB/s).
+constexpr int kSlideAhead = 8;
+
 __global__ void __launch_bounds__(256) xy_slide_kernel(const __grid_constant__ XySlideParams c) {
   extern __shared__ __align__(16) unsigned char smem[];
-  float2* w = reinterpret_cast<float2*>(smem);
-  for (int k = threadIdx.x; k < c.nl; k += blockDim.x) w[k] = ldg2(c.wq + k);
+  float2* w = reinterpret_cast<float2*>(smem);  // the slots' factors exp(-2 pi i z0 t / nl), in the order they are read
+  for (int j = threadIdx.x; j < c.k; j += blockDim.x) w[j] = ldg2(c.wq + (int)((long long)c.z0 * ((c.slot0 + j) % c.nl) % c.nl));
   __syncthreads();
-  const size_t row = (size_t)c.ntx * kTile;
-  const size_t n = (size_t)c.wy * row;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int kyw = (int)(i / row), tile = (int)(i % row) / kTile, pix = (int)(i % kTile);
-    const int kxw = tile * kTile + pix;
-    const float2* h = c.inter + ((size_t)kyw * c.ntx + tile) * c.nl * kTile + pix;
-    float2 d = make_float2(0.f, 0.f);
-    int t = c.slot0;
-    for (int j = 0; j < c.k; ++j) {
-      const float2 v = __ldcs(h + (size_t)t * kTile);
-      const float2 e = w[(c.z0 * t) % c.nl];
-      d.x = fmaf(v.x, e.x, fmaf(-v.y, e.y, d.x));
-      d.y = fmaf(v.x, e.y, fmaf(v.y, e.x, d.y));
+  const size_t pairs = (size_t)c.wy * c.ntx * (kTile / 2);
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= pairs) return;
+  const size_t tile = i / (kTile / 2);  // kyw * ntx + tile of the row
+  const int pix = 2 * (int)(i % (kTile / 2));
+  const float4* h = reinterpret_cast<const float4*>(c.inter + tile * c.nl * kTile + pix);  // slot t at h + t * kTile / 2
+  float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+  int t = c.slot0;
+  for (int j0 = 0; j0 < c.k; j0 += kSlideAhead) {
+    float4 v[kSlideAhead];
+#pragma unroll
+    for (int j = 0; j < kSlideAhead; ++j) {
+      if (j0 + j < c.k) v[j] = __ldcs(h + (size_t)t * (kTile / 2));
       if (++t == c.nl) t = 0;
     }
-    float2 acc = c.state[i];
-    acc.x = fmaf(c.sign, d.x, acc.x);
-    acc.y = fmaf(c.sign, d.y, acc.y);
-    c.state[i] = acc;
-    if (c.xy && kxw < c.wx) c.xy[(size_t)kyw * c.wx + kxw] = envelope(acc, c.power_scale, c.magnitude);
+#pragma unroll
+    for (int j = 0; j < kSlideAhead; ++j)
+      if (j0 + j < c.k) {
+        const float2 e = w[j0 + j];
+        d.x = fmaf(v[j].x, e.x, fmaf(-v[j].y, e.y, d.x));
+        d.y = fmaf(v[j].x, e.y, fmaf(v[j].y, e.x, d.y));
+        d.z = fmaf(v[j].z, e.x, fmaf(-v[j].w, e.y, d.z));
+        d.w = fmaf(v[j].z, e.y, fmaf(v[j].w, e.x, d.w));
+      }
   }
+  float4* st = reinterpret_cast<float4*>(c.state) + i;
+  float4 acc = *st;
+  acc.x = fmaf(c.sign, d.x, acc.x);
+  acc.y = fmaf(c.sign, d.y, acc.y);
+  acc.z = fmaf(c.sign, d.z, acc.z);
+  acc.w = fmaf(c.sign, d.w, acc.w);
+  *st = acc;
+  if (!c.xy) return;
+  const int kyw = (int)(tile / c.ntx), kxw = (int)(tile - (size_t)kyw * c.ntx) * kTile + pix;
+  float* xy = c.xy + (size_t)kyw * c.wx + kxw;
+  if (kxw < c.wx) xy[0] = envelope(make_float2(acc.x, acc.y), c.power_scale, c.magnitude);
+  if (kxw + 1 < c.wx) xy[1] = envelope(make_float2(acc.z, acc.w), c.power_scale, c.magnitude);
 }
 
-// xz and yz cuts: the axial kernel's transform on the tiles of row y0 (blocks
-// 0 .. ntx-1) and on the tile holding column x0 of every row (the next wy
-// blocks), keeping only the cut's pixels.
+// xz and yz cuts: the axial kernels' transform (the same split and the same
+// arithmetic per pixel, so the cuts equal the volume's bit for bit) on lines of
+// kLinePix pixels: row y0 of the window (the first blocks), then column x0.  A
+// pixel of the column lies in a tile of its own, and only its 32-byte sectors
+// are read: transforming whole tiles for one column of them read 64 MB instead
+// of 8 at 1024 x 1024 x 256.  Eight pixels a block give 256 blocks there.
+constexpr int kLinePix = 8;
+
 template <int NL>
-__global__ void __launch_bounds__(kTile * Split<NL>::N1) gate_lines_kernel(const __grid_constant__ GateCutsParams c) {
-  constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
+__global__ void __launch_bounds__(kLinePix * ax_split_n1(NL)) gate_lines_kernel(const __grid_constant__ GateCutsParams c) {
+  constexpr int N1 = ax_split_n1(NL), N2 = NL / N1, P = kLinePix;
+  using S2 = Stage2<NL, N1>;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* ex = reinterpret_cast<float2*>(smem);
-  const bool xz_block = (int)blockIdx.x < c.ntx;
-  const int kyw = xz_block ? c.y0 : (int)blockIdx.x - c.ntx;
-  const int tile = xz_block ? (int)blockIdx.x : c.x0 / kTile;
-  const int pix = threadIdx.x % kTile, j1 = threadIdx.x / kTile;
-  const float2* src = c.inter + ((size_t)kyw * c.ntx + tile) * NL * kTile + pix;
-  float2 a[N2];
+  const int xz_blocks = c.xz ? (c.wx + P - 1) / P : 0;
+  const bool xz_block = (int)blockIdx.x < xz_blocks;
+  const int pix = threadIdx.x % P, j1 = threadIdx.x / P;
+  const int at = (xz_block ? (int)blockIdx.x : (int)blockIdx.x - xz_blocks) * P + pix;  // along the line
+  const bool in = at < (xz_block ? c.wx : c.wy);
+  const int kxw = xz_block ? at : c.x0, kyw = xz_block ? c.y0 : at;
+  float2 a[S2::A];
+  if (in) {
+    const float2* src = c.inter + ((size_t)kyw * c.ntx + kxw / kTile) * NL * kTile + kxw % kTile;
 #pragma unroll
-  for (int j2 = 0; j2 < N2; ++j2) a[j2] = __ldcs(src + (j1 + N1 * j2) * kTile);
+    for (int j2 = 0; j2 < N2; ++j2) a[j2] = __ldcs(src + (j1 + N1 * j2) * kTile);
+  } else {
+#pragma unroll
+    for (int j2 = 0; j2 < N2; ++j2) a[j2] = make_float2(0.f, 0.f);
+  }
   Dft<N2, -1>::template run<1, 0>(a);
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) a[k2] = cmul(a[k2], ldg2(c.twl + k2 * N1 + j1));
 #pragma unroll
-  for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * kTile + pix] = a[k2];
+  for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * P + pix] = a[k2];
   __syncthreads();
-  static_for<0, N2 / N1>([&](auto I) {
+  static_for<0, S2::NI>([&](auto I) {
     constexpr int i = decltype(I)::value;
     const int k2 = j1 + N1 * i;
+    if (!S2::live(i, j1)) return;
 #pragma unroll
-    for (int jj = 0; jj < N1; ++jj) a[i * N1 + jj] = ex[(k2 * N1 + jj) * kTile + pix];
+    for (int jj = 0; jj < N1; ++jj) a[i * N1 + jj] = ex[(k2 * N1 + jj) * P + pix];
     Dft<N1, -1>::template run<1, i * N1>(a);
   });
-  const int kxw = tile * kTile + pix;
-  if (kxw >= c.wx) return;
-  if (xz_block ? !c.xz : (!c.yz || kxw != c.x0)) return;
-  static_for<0, N2 / N1>([&](auto I) {
+  if (!in) return;
+  static_for<0, S2::NI>([&](auto I) {
     constexpr int i = decltype(I)::value;
     const int k2 = j1 + N1 * i;
+    if (!S2::live(i, j1)) return;
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) {
       const int q = k2 + N2 * k1;
@@ -666,10 +725,9 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) gate_lines_kernel(const
 
 template <int NL>
 cudaError_t launch_lines(const GateCutsParams& c, cudaStream_t s) {
-  const size_t smem = (size_t)NL * kTile * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(gate_lines_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  gate_lines_kernel<NL><<<c.ntx + c.wy, kTile * Split<NL>::N1, smem, s>>>(c);
+  const size_t smem = (size_t)NL * kLinePix * sizeof(float2);  // at most 32 KB
+  const int blocks = (c.xz ? (c.wx + kLinePix - 1) / kLinePix : 0) + (c.yz ? (c.wy + kLinePix - 1) / kLinePix : 0);
+  gate_lines_kernel<NL><<<blocks, kLinePix * ax_split_n1(NL), smem, s>>>(c);
   return cudaGetLastError();
 }
 
@@ -699,33 +757,38 @@ cudaError_t launch_ra_tiles(const RescaleAxialTileParams& rp, const CUtensorMap&
 template <int NL>
 cudaError_t launch_stream(const AxialParams& ap, int num_sms, cudaStream_t s) {
   using S = AxStream<NL>;
-  const size_t smem = (size_t)S::kStages * S::kTileBytes;
+  const size_t smem = (size_t)S::kStages * S::kUnitBytes;
+  alignas(64) CUtensorMap imap = {};
+  if (S::kUnits > 1 && !encode_inter_map(ap.inter, (long long)ap.ntx * ap.wy * NL, S::kPix, &imap))
+    return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(axial_stream_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, axial_stream_kernel<NL>, S::kThreadsAll, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const long long ntiles = (long long)ap.ntx * ap.wy;
+  const long long nunits = (long long)ap.ntx * ap.wy * S::kUnits;
   long long grid = (long long)(num_sms > 0 ? num_sms : 1) * per_sm;
-  if (grid > ntiles) grid = ntiles;
+  if (grid > nunits) grid = nunits;
   if (grid < 1) return cudaSuccess;
-  axial_stream_kernel<NL><<<(unsigned)grid, S::kThreadsAll, smem, s>>>(ap);
+  axial_stream_kernel<NL><<<(unsigned)grid, S::kThreadsAll, smem, s>>>(ap, imap);
   return cudaGetLastError();
 }
 
 template <int NL>
 cudaError_t launch(const AxialParams& ap, int num_sms, cudaStream_t s) {
-  // the streaming form where a tile fits a third of the ring and a group has
-  // eight warps or more; otherwise one CTA per tile
-  constexpr bool kStream = (size_t)NL * kTile * sizeof(float2) <= 64 * 1024 && kTile * split_n1(NL) >= 256;
-  if constexpr (kStream) return launch_stream<NL>(ap, num_sms, s);
-  const size_t smem = (size_t)NL * kTile * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(axial_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(ap.ntx, ap.wy);
-  axial_kernel<NL><<<grid, kTile * Split<NL>::N1, smem, s>>>(ap);
-  return cudaGetLastError();
+  // the streaming form from 64 frames on; tiles of 16 and 32 frames (4 and 8 KB)
+  // are smaller than a hand-over is worth, and take one CTA each
+  if constexpr (NL >= 64) {
+    return launch_stream<NL>(ap, num_sms, s);
+  } else {
+    const size_t smem = (size_t)NL * kTile * sizeof(float2);
+    cudaError_t e = cudaFuncSetAttribute(axial_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid(ap.ntx, ap.wy);
+    axial_kernel<NL><<<grid, kTile * Split<NL>::N1, smem, s>>>(ap);
+    return cudaGetLastError();
+  }
 }
 
 #define SSOCT_AXIAL_SIZES(X) X(16) X(32) X(64) X(96) X(128) X(160) X(200) X(256) X(512)
@@ -743,7 +806,8 @@ cudaError_t launch_xy_slide(const Plan& p, int slot0, int k, int z0, float sign,
   c.sign = sign;
   c.power_scale = (float)(p.alpha * p.alpha);
   c.magnitude = (p.flags & SSOCT_FLAG_MAGNITUDE) ? 1 : 0;
-  xy_slide_kernel<<<4 * p.num_sms, 256, (size_t)p.nl * sizeof(float2), s>>>(c);
+  const size_t pairs = (size_t)p.wy * p.ntx * (kTile / 2);
+  xy_slide_kernel<<<(unsigned)((pairs + 255) / 256), 256, (size_t)std::max(k, 1) * sizeof(float2), s>>>(c);
   return cudaGetLastError();
 }
 
@@ -752,7 +816,7 @@ cudaError_t launch_gate_cuts(const Plan& p, int x0, int y0, int z0, float* xy, f
   GateCutsParams c;
   c.inter = (const float2*)(p.ws + p.off_inter);
   c.wq = (const float2*)(p.ws + p.off_wq);
-  c.twl = (const float2*)(p.ws + p.off_twl);
+  c.twl = (const float2*)(p.ws + p.off_twax);
   c.xy = xy;
   c.xz = xz;
   c.yz = yz;

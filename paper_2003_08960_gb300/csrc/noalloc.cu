@@ -121,6 +121,7 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
       {p.off_twx, p.twx.data(), sizeof(float2) * p.twx.size()},
       {p.off_twy, p.twy.data(), sizeof(float2) * p.twy.size()},
       {p.off_twl, p.twl.data(), sizeof(float2) * p.twl.size()},
+      {p.off_twax, p.twax.data(), sizeof(float2) * p.twax.size()},
       {p.off_tcb, p.tcb.data(), sizeof(unsigned short) * p.tcb.size()},
   };
   for (const Up& u : ups) {
@@ -187,7 +188,7 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   ap.inter = lp.inter;
   ap.vol = vol_dev;
   ap.cplx = (float2*)complex_dev;
-  ap.twl = (const float2*)(ws + p.off_twl);
+  ap.twl = (const float2*)(ws + p.off_twax);
   ap.ox = (const float2*)(ws + p.off_ox);
   ap.oy = (const float2*)(ws + p.off_oy);
   ap.nl = p.nl; ap.wx = p.wx; ap.wy = p.wy; ap.ntx = p.ntx;

@@ -782,7 +782,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     ap.inter = p.inter;
     ap.vol = vol;
     ap.cplx = nullptr;
-    ap.twl = p.twl;
+    ap.twl = (const float2*)(ws + pl.off_twax);
     ap.ox = (const float2*)(ws + pl.off_ox);
     ap.oy = (const float2*)(ws + pl.off_oy);
     ap.nl = pl.nl; ap.wx = pl.wx; ap.wy = pl.wy; ap.ntx = pl.ntx;

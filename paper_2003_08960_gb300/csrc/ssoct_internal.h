@@ -43,6 +43,14 @@ __host__ __device__ constexpr int ra_split_n1(int nl) {
   return nl == 96 ? 16 : nl == 160 ? 16 : nl == 200 ? 20 : split_n1(nl);
 }
 
+// Split of the sweep transform in the axial kernels that write volumes and cuts:
+// 8 x 12, 8 x 20 and 10 x 20 for 96, 160 and 200 frames, whose general splits
+// (4 x 24, 4 x 40, 5 x 40) would leave four or five warps per tile and 24 or 40
+// values per thread.
+__host__ __device__ constexpr int ax_split_n1(int nl) {
+  return nl == 96 ? 8 : nl == 160 ? 8 : nl == 200 ? 10 : split_n1(nl);
+}
+
 // Rows per tensor copy of a lateral column band: the largest divisor of ny up
 // to 256 (a box dimension's limit), so that whole boxes cover the column.
 __host__ __device__ constexpr int band_box_rows(int ny) {
@@ -206,7 +214,7 @@ struct AxialParams {
   const float2* inter;     // [wy][ntx][nl][32]
   float* vol;              // [nl][wy][wx]
   float2* cplx;            // optional [nl][wy][wx]
-  const float2* twl;       // [N2l][N1l], sign -
+  const float2* twl;       // [N2][N1] of ax_split_n1, sign -
   const float2* ox;        // [wx] output chirp (x), incl. centring phase
   const float2* oy;        // [wy] output chirp (y) times the prefactor K
   int nl, wx, wy, ntx;
@@ -234,7 +242,7 @@ struct Plan {
   double alpha;             // d^2 / (lambda_1 z) = |K|
   // host tables
   std::vector<Tap> xtab, ytab;
-  std::vector<float2> cx, cy, cx2, cy2, ox, oy, twx, twy, twl, twra;
+  std::vector<float2> cx, cy, cx2, cy2, ox, oy, twx, twy, twl, twra, twax;
   std::vector<float2> wq;   // [nl] exp(-2 pi i k / nl), for single-bin transforms
   std::vector<unsigned short> tcb;  // SSOCT_FLAG_TC_AXIAL: BF16 hi / lo 16-point DFT matrix (operand layout)
   // SSOCT_FLAG_PUPIL: input chirp x Zernike screen, its distance z and |K|, frames per Q chunk
@@ -257,6 +265,7 @@ struct Plan {
   // workspace layout (byte offsets)
   size_t off_ctr, off_xtab, off_ytab, off_cx, off_cy, off_cx2, off_cy2, off_ox, off_oy, off_twx, off_twy, off_twl;
   size_t off_twra = 0;       // twiddles of the tiled first pass's split (ra_split_n1)
+  size_t off_twax = 0;       // twiddles of the axial kernels' split (ax_split_n1; off_twl where the splits agree)
   size_t off_tcb, off_wq, off_ring, off_scratch, off_inter, ws_bytes;
   size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0, off_cis = 0;  // SSOCT_FLAG_PUPIL regions
   // Frame sizes the persistent lateral kernel does not compile (384, 640, 768)
