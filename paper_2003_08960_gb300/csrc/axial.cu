@@ -94,7 +94,9 @@ struct AxStream {
   using S2 = Stage2<NL, N1>;
   static constexpr int kPix = NL > 256 ? kTile / 2 : kTile;
   static constexpr int kUnits = kTile / kPix;  // per tile
-  static constexpr int kGroups = NL == 96 ? 4 : NL == 160 ? 3 : 2;
+  // three groups where a unit is short (1024 x 1024 x 64: two 150 us, three 130,
+  // four 131; 128 frames: two 151, three 153, four 154 at 768 x 768)
+  static constexpr int kGroups = NL == 64 || NL == 96 || NL == 160 ? 3 : 2;
   static constexpr int kGroupThreads = kPix * N1;
   static constexpr int kThreadsAll = kGroups * kGroupThreads;
   static constexpr size_t kUnitBytes = (size_t)NL * kPix * sizeof(float2);

@@ -67,6 +67,21 @@ cudaError_t scratch_on_device(int dev, char** addr, int* sms) {
   return cudaSuccess;
 }
 
+// Taps of Eq. 5 of every frame and axis from the rescale ratios, and zeroed work
+// counters.  Every call needs the taps anew, and building them here takes 2 us
+// where their upload (0.5 MB from pageable memory at 256 x 256 x 64, ten small
+// tables beside it) took 35 us of the call's 85.
+__global__ void __launch_bounds__(256) noalloc_tables_kernel(Tap* xtab, Tap* ytab, const double* ratio, int nx, int ny,
+                                                             int nl, unsigned* counters, int ncounters) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < ncounters) counters[i] = 0u;
+  const int per = nx + ny;
+  if (i >= nl * per) return;
+  const int t = i / per, k = i - t * per;
+  if (k < nx) xtab[t * nx + k] = eq5_tap(k, nx, ratio[t]);
+  else ytab[t * ny + k - nx] = eq5_tap(k - nx, ny, ratio[t]);
+}
+
 ssoct_status fail(Plan& p, ssoct_status s, const std::string& msg) {
   p.last_error = msg;
   return s;
@@ -106,31 +121,16 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   cudaStream_t s = (cudaStream_t)stream;
 
   // Tables of this plan (the previous call may have left another plan's), then
-  // zeroed work counters.
-  struct Up {
-    size_t off;
-    const void* src;
-    size_t n;
-  } ups[] = {
-      {p.off_xtab, p.xtab.data(), sizeof(Tap) * p.xtab.size()},
-      {p.off_ytab, p.ytab.data(), sizeof(Tap) * p.ytab.size()},
-      {p.off_cx, p.cx.data(), sizeof(float2) * p.cx.size()},
-      {p.off_cy, p.cy.data(), sizeof(float2) * p.cy.size()},
-      {p.off_ox, p.ox.data(), sizeof(float2) * p.ox.size()},
-      {p.off_oy, p.oy.data(), sizeof(float2) * p.oy.size()},
-      {p.off_twx, p.twx.data(), sizeof(float2) * p.twx.size()},
-      {p.off_twy, p.twy.data(), sizeof(float2) * p.twy.size()},
-      {p.off_twl, p.twl.data(), sizeof(float2) * p.twl.size()},
-      {p.off_twax, p.twax.data(), sizeof(float2) * p.twax.size()},
-      {p.off_tcb, p.tcb.data(), sizeof(unsigned short) * p.tcb.size()},
-  };
-  for (const Up& u : ups) {
-    if (!u.n) continue;
-    e = cudaMemcpyAsync(ws + u.off, u.src, u.n, cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return fail(p, SSOCT_ECUDA, std::string("table upload: ") + cudaGetErrorString(e));
-  }
-  e = cudaMemsetAsync(ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
-  if (e != cudaSuccess) return fail(p, SSOCT_ECUDA, std::string("counter reset: ") + cudaGetErrorString(e));
+  // the taps of Eq. 5 and zeroed work counters.
+  e = cudaMemcpyAsync(ws + p.off_image, p.image.data(), p.image.size(), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return fail(p, SSOCT_ECUDA, std::string("table upload: ") + cudaGetErrorString(e));
+  const int counters = (int)(sizeof(Counters) / sizeof(unsigned)) + 2 * p.nl;
+  const int taps = p.nl * (p.nx + p.ny);
+  noalloc_tables_kernel<<<(std::max(taps, counters) + 255) / 256, 256, 0, s>>>(
+      (Tap*)(ws + p.off_xtab), (Tap*)(ws + p.off_ytab), (const double*)(ws + p.off_ratio), p.nx, p.ny, p.nl,
+      (unsigned*)(ws + p.off_ctr), counters);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(p, SSOCT_ECUDA, std::string("tables kernel launch: ") + cudaGetErrorString(e));
   if (p.inject_skip) {
     // start the ticket counter past the first items (ssoct_inject_stall); the
     // copy reads the plan's own field, and the sync keeps it a test-only cost

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <string>
@@ -68,6 +69,29 @@ struct __align__(16) Tap {
   float w1;
   float pad;
 };
+
+// Eq. 5 along one axis: output pixel i reads the input at u = c + (i - c) s,
+// c = n / 2, by linear interpolation; a tap outside [0, n) reads 0.
+__host__ __device__ inline Tap eq5_tap(int i, int n, double s) {
+  const double c = n / 2.0;
+  const double u = c + (i - c) * s;
+  const double fl = floor(u);
+  const double a = u - fl;
+  const long long i0 = (long long)fl, i1 = i0 + 1;
+  const double w0 = (i0 >= 0 && i0 < n) ? 1.0 - a : 0.0;
+  const double w1 = (i1 >= 0 && i1 < n) ? a : 0.0;
+  long long b = i0 < 0 ? 0 : i0;
+  if (b > n - 2) b = n - 2;
+  double wb = 0.0, wb1 = 0.0;
+  if (i0 == b) wb += w0; else if (i0 == b + 1) wb1 += w0;
+  if (i1 == b) wb += w1; else if (i1 == b + 1) wb1 += w1;
+  Tap t;
+  t.base = (int)b;
+  t.w0 = (float)wb;
+  t.w1 = (float)wb1;
+  t.pad = 0.f;
+  return t;
+}
 
 // Eq. 5 along a 64-pixel strip x0 .. x0 + 63 of one frame (axial-first order):
 // the position u(x0 + k) = u(x0) + k s_t lies at staged column
@@ -266,8 +290,13 @@ struct Plan {
   size_t off_ctr, off_xtab, off_ytab, off_cx, off_cy, off_cx2, off_cy2, off_ox, off_oy, off_twx, off_twy, off_twl;
   size_t off_twra = 0;       // twiddles of the tiled first pass's split (ra_split_n1)
   size_t off_twax = 0;       // twiddles of the axial kernels' split (ax_split_n1; off_twl where the splits agree)
+  size_t off_cis = 0;        // exp(i pi k / 128) (pupil_cis_table)
+  // host image of the workspace from off_image on (the tables but the taps), and
+  // the rescale ratios lambda_t / lambda_1 in it
+  std::vector<unsigned char> image;
+  size_t off_image = 0, off_ratio = 0;
   size_t off_tcb, off_wq, off_ring, off_scratch, off_inter, ws_bytes;
-  size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0, off_cis = 0;  // SSOCT_FLAG_PUPIL regions
+  size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0;  // SSOCT_FLAG_PUPIL regions
   // Frame sizes the persistent lateral kernel does not compile (384, 640, 768)
   // take the two-pass lateral path of sharpness.cu: chirp table and frame buffer.
   bool generic = false;

@@ -40,29 +40,6 @@ float2 cis_pi(double r) {
   return make_float2((float)std::cos(a), (float)std::sin(a));
 }
 
-// Eq. 5 along one axis: output pixel i reads the input at u = c + (i - c) s,
-// c = n / 2, by linear interpolation; a tap outside [0, n) reads 0.
-Tap make_tap(int i, int n, double s) {
-  const double c = n / 2.0;
-  const double u = c + (i - c) * s;
-  const double fl = std::floor(u);
-  const double a = u - fl;
-  const long i0 = (long)fl, i1 = i0 + 1;
-  const double w0 = (i0 >= 0 && i0 < n) ? 1.0 - a : 0.0;
-  const double w1 = (i1 >= 0 && i1 < n) ? a : 0.0;
-  long b = i0 < 0 ? 0 : i0;
-  if (b > n - 2) b = n - 2;
-  double wb = 0.0, wb1 = 0.0;
-  if (i0 == b) wb += w0; else if (i0 == b + 1) wb1 += w0;
-  if (i1 == b) wb += w1; else if (i1 == b + 1) wb1 += w1;
-  Tap t;
-  t.base = (int)b;
-  t.w0 = (float)wb;
-  t.w1 = (float)wb1;
-  t.pad = 0.f;
-  return t;
-}
-
 // Input chirp of Eq. 6 times the centring phase along one axis of length n:
 // exp(-i pi [(k - n/2)^2 alpha + k]); alpha = d^2 / (lambda_1 z).  With it the
 // centred sum over (k - n/2)(m - n/2) / n becomes a plain DFT over k m / n.
@@ -246,8 +223,8 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.ytab.resize((size_t)nlambda * ny);
   for (int t = 0; t < nlambda; ++t) {
     const double s = lambda_m[t] / p.lambda1;
-    for (int i = 0; i < nx; ++i) p.xtab[(size_t)t * nx + i] = make_tap(i, nx, s);
-    for (int j = 0; j < ny; ++j) p.ytab[(size_t)t * ny + j] = make_tap(j, ny, s);
+    for (int i = 0; i < nx; ++i) p.xtab[(size_t)t * nx + i] = eq5_tap(i, nx, s);
+    for (int j = 0; j < ny; ++j) p.ytab[(size_t)t * ny + j] = eq5_tap(j, ny, s);
   }
   // Axial-first order, tiled first pass: one strip record per (frame, 64-pixel
   // strip), and the staged width that holds every frame's taps of a strip
@@ -361,6 +338,10 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.off_ctr = take(sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)nlambda);
   p.off_xtab = take(sizeof(Tap) * p.xtab.size());
   p.off_ytab = take(sizeof(Tap) * p.ytab.size());
+  const size_t before_cis = off;
+  p.off_cis = take(sizeof(float4) * 256);  // used with SSOCT_FLAG_PUPIL; every plan has its place
+  const size_t first_table = off;
+  size_t beside = off - before_cis;  // bytes that the no-allocation path's size limit leaves out
   p.off_cx = take(sizeof(float2) * nx);
   p.off_cy = take(sizeof(float2) * ny);
   p.off_cx2 = take(sizeof(float2) * nx);
@@ -370,10 +351,39 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.off_twx = take(sizeof(float2) * p.twx.size());
   p.off_twy = take(sizeof(float2) * p.twy.size());
   p.off_twl = take(sizeof(float2) * p.twl.size());
+  const size_t before_twax = off;
   p.off_twax = p.twax.empty() ? p.off_twl : take(sizeof(float2) * p.twax.size());
+  beside += off - before_twax;
   p.off_twra = take(sizeof(float2) * p.twra.size());
   p.off_tcb = take(sizeof(unsigned short) * p.tcb.size());
   p.off_wq = take(sizeof(float2) * p.wq.size());
+  const size_t before_ratio = off;
+  p.off_ratio = take(sizeof(double) * nlambda);
+  beside += off - before_ratio;
+  // the tables from off_cx on, as one image of the workspace's bytes
+  p.off_image = first_table;
+  p.image.assign(off - first_table, 0);
+  {
+    auto put = [&](size_t at, const void* src, size_t bytes) {
+      if (bytes) memcpy(p.image.data() + (at - first_table), src, bytes);
+    };
+    std::vector<double> ratio(nlambda);
+    for (int t = 0; t < nlambda; ++t) ratio[t] = lambda_m[t] / p.lambda1;
+    put(p.off_cx, p.cx.data(), sizeof(float2) * p.cx.size());
+    put(p.off_cy, p.cy.data(), sizeof(float2) * p.cy.size());
+    put(p.off_cx2, p.cx2.data(), sizeof(float2) * p.cx2.size());
+    put(p.off_cy2, p.cy2.data(), sizeof(float2) * p.cy2.size());
+    put(p.off_ox, p.ox.data(), sizeof(float2) * p.ox.size());
+    put(p.off_oy, p.oy.data(), sizeof(float2) * p.oy.size());
+    put(p.off_twx, p.twx.data(), sizeof(float2) * p.twx.size());
+    put(p.off_twy, p.twy.data(), sizeof(float2) * p.twy.size());
+    put(p.off_twl, p.twl.data(), sizeof(float2) * p.twl.size());
+    put(p.off_twax, p.twax.data(), sizeof(float2) * p.twax.size());
+    put(p.off_twra, p.twra.data(), sizeof(float2) * p.twra.size());
+    put(p.off_tcb, p.tcb.data(), sizeof(unsigned short) * p.tcb.size());
+    put(p.off_wq, p.wq.data(), sizeof(float2) * p.wq.size());
+    put(p.off_ratio, ratio.data(), sizeof(double) * ratio.size());
+  }
   p.off_ring = take(sizeof(uint16_t) * (size_t)nlambda * ny * nx);
   p.off_scratch = take(generic ? 0 : sizeof(float2) * (size_t)p.slots_alloc * ny * p.wxp);
   const size_t inter_bytes = sizeof(float2) * (size_t)p.wy * p.ntx * nlambda * kTile;
@@ -395,10 +405,10 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     p.off_cp = take(sizeof(float2) * (size_t)nx * ny);
     p.off_Q = take(sizeof(float2) * chunks * ny * nx);
     p.off_red = take(sizeof(double) * kShRedDoubles);
-    p.off_cis = take(sizeof(float4) * 256);
   }
   p.ws_bytes = off;
-  p.noalloc_bytes = generic ? off : off - sizeof(float2) * (size_t)(p.slots_alloc - p.slots_noalloc) * ny * p.wxp;
+  p.noalloc_bytes = off - beside;
+  if (!generic) p.noalloc_bytes -= sizeof(float2) * (size_t)(p.slots_alloc - p.slots_noalloc) * ny * p.wxp;
   *out = h;
   return SSOCT_OK;
 }
@@ -442,19 +452,7 @@ ssoct_status ssoct_set_workspace(ssoct_plan h, void* dev_ptr, size_t bytes) {
   struct Up { size_t off; const void* src; size_t n; } ups[] = {
       {p.off_xtab, p.xtab.data(), sizeof(Tap) * p.xtab.size()},
       {p.off_ytab, p.ytab.data(), sizeof(Tap) * p.ytab.size()},
-      {p.off_cx, p.cx.data(), sizeof(float2) * p.cx.size()},
-      {p.off_cy, p.cy.data(), sizeof(float2) * p.cy.size()},
-      {p.off_cx2, p.cx2.data(), sizeof(float2) * p.cx2.size()},
-      {p.off_cy2, p.cy2.data(), sizeof(float2) * p.cy2.size()},
-      {p.off_ox, p.ox.data(), sizeof(float2) * p.ox.size()},
-      {p.off_oy, p.oy.data(), sizeof(float2) * p.oy.size()},
-      {p.off_twx, p.twx.data(), sizeof(float2) * p.twx.size()},
-      {p.off_twy, p.twy.data(), sizeof(float2) * p.twy.size()},
-      {p.off_twl, p.twl.data(), sizeof(float2) * p.twl.size()},
-      {p.off_twax, p.twax.data(), sizeof(float2) * p.twax.size()},
-      {p.off_twra, p.twra.data(), sizeof(float2) * p.twra.size()},
-      {p.off_tcb, p.tcb.data(), sizeof(unsigned short) * p.tcb.size()},
-      {p.off_wq, p.wq.data(), sizeof(float2) * p.wq.size()},
+      {p.off_image, p.image.data(), p.image.size()},
       {p.off_xstrip, p.xstrip.data(), sizeof(StripTap) * p.xstrip.size()},
   };
   for (const Up& u : ups) {
