@@ -784,9 +784,7 @@ cudaError_t launch(const AxialParams& ap, int num_sms, cudaStream_t s) {
   if constexpr (NL >= 64) {
     return launch_stream<NL>(ap, num_sms, s);
   } else {
-    const size_t smem = (size_t)NL * kTile * sizeof(float2);
-    cudaError_t e = cudaFuncSetAttribute(axial_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)NL * kTile * sizeof(float2);  // at most 8 KB
     dim3 grid(ap.ntx, ap.wy);
     axial_kernel<NL><<<grid, kTile * Split<NL>::N1, smem, s>>>(ap);
     return cudaGetLastError();

@@ -281,6 +281,7 @@ struct Plan {
   int rows_per_item, cols_per_item;
   int wxp, ntx;
   int stage_rows;
+  int small_rows = 0;        // see lateral_small_rows
   LateralSchedule sch;
   int slots_alloc = 0;       // scratch-ring slots the workspace holds (sch.slots <= slots_alloc)
   int slots_noalloc = 0;     // ring slots counted in noalloc_bytes
@@ -370,6 +371,11 @@ bool encode_frames_map(const Plan& p, const uint16_t* frames, int box_cols, void
 // complex values x 256 rows.
 bool encode_inter_map(const float2* inter, long long rows, int box_complex, void* map_out);
 bool lateral_supported(int nx, int ny);
+// Frames that one CTA or cluster transforms whole, without the work queue: the
+// raw rows that a CTA's band takes (0: not such a plan), and whether the next
+// launch goes that way.
+int lateral_small_rows(const Plan& p);
+bool lateral_small(const Plan& p);
 bool axial_supported(int nl);
 // Tensor-core axial kernel (axial_tc.cu): sweep lengths it handles, its DFT
 // operand table, dynamic shared memory, and launcher.  err is the plan's error

@@ -327,6 +327,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
       if (rows > st) st = rows;
     }
   p.stage_rows = st;
+  p.small_rows = lateral_small_rows(p);
   if (!generic && lateral_smem_bytes(p) > 227u * 1024u) {
     delete h;
     return SSOCT_EUNSUPPORTED;  // rescale ratio too far from 1 for the staging buffer
@@ -571,7 +572,10 @@ static LateralParams lateral_params(const Plan& p, const uint16_t* frames, int r
 // of ssoct_profile); *ev receives the event slots of this call, if profiling.
 static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaStream_t s, cudaEvent_t** ev) {
   char* ws = p.ws;
-  cudaError_t e = cudaMemsetAsync(ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
+  // the work queue's counters; paths without a queue leave the error word to ssoct_sync
+  cudaError_t e = cudaSuccess;
+  if (!p.generic && !lateral_small(p))
+    e = cudaMemsetAsync(ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
   if (p.inject_skip) {
     // start the ticket counter past the first items (ssoct_inject_stall)
