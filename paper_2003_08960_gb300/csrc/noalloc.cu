@@ -159,7 +159,7 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   if (!encode_scratch_map_at(p, scratch, room, tmap))
     return fail(p, SSOCT_ECUDA, "cuTensorMapEncodeTiled failed for the no-allocation scratch ring");
 
-  LateralParams lp;
+  LateralParams lp = {};
   lp.frames = frames_dev;
   lp.ring_start = 0;
   lp.tab0 = 0;

@@ -744,7 +744,7 @@ cudaError_t launch_lateral_generic(const Plan& pl, const uint16_t* frames, int r
   return e;
 }
 
-cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, cudaStream_t s) {
+cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, bool have_inter, cudaStream_t s) {
   char* ws = pl.ws;
   ShParams p = {};
   p.frames = frames;
@@ -775,8 +775,8 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   const int chunks = (pl.nl + pl.sh_tpc - 1) / pl.sh_tpc;
 
   cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
-  if (e == cudaSuccess) e = rows_any(false, p, chunks, s);
-  if (e == cudaSuccess) e = cols_any(false, p, s);
+  if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
+  if (e == cudaSuccess && !have_inter) e = cols_any(false, p, s);
   if (e == cudaSuccess) {
     AxialParams ap;
     ap.inter = p.inter;

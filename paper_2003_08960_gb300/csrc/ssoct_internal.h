@@ -222,6 +222,7 @@ struct LateralParams {
   LateralSchedule sch;
   int stage_rows;          // input rows staged per row item (max over items)
   int stage_bytes;         // bytes of one shared-memory stage buffer (set at launch)
+  const float2* cp;        // [ny][nx] chirp x pupil screen in the place of cx, cy, or NULL
   unsigned long long wait_ns;  // limit of every device-side wait (0 = default)
   // axial-first order (SSOCT_FLAG_AXIAL_FIRST): frame f is depth bin af_bin(f);
   // row items read half-spectrum planes, column items write the volume
@@ -282,6 +283,8 @@ struct Plan {
   int wxp, ntx;
   int stage_rows;
   int small_rows = 0;        // see lateral_small_rows
+  bool pair_queue = false;   // generic plans: launch_lateral_pair takes the plan's frames
+  bool pupil_queue = false;  // aberration path: launch_lateral_pupil does
   LateralSchedule sch;
   int slots_alloc = 0;       // scratch-ring slots the workspace holds (sch.slots <= slots_alloc)
   int slots_noalloc = 0;     // ring slots counted in noalloc_bytes
@@ -398,10 +401,21 @@ cudaError_t launch_lateral_generic(const Plan& pl, const uint16_t* frames, int r
 void build_pupil_table(int nx, int ny, double alpha, const double* coeffs, int ncoeffs, std::vector<float2>& out);
 // exp(i pi k / 128), k = 0 .. 255, as pairs of floats (re hi, re lo, im hi, im lo).
 void pupil_cis_table(std::vector<float4>& out);
-cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, cudaStream_t s);
+// have_inter: the sweep-axis intermediate already holds the holograms of the frames.
+cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, bool have_inter, cudaStream_t s);
 cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s);
 // Dynamic shared memory of the lateral kernel for a plan (bytes).
 size_t lateral_smem_bytes(const Plan& p);
+// The lateral kernel's instances in units of their own: square frames of 640 and
+// more; non-square frames by width (paper order); square frames with the table
+// lp.cp for the chirp (aberration path).
+cudaError_t launch_lateral_large(const Plan& p, const LateralParams& lp, const void* tmap, int num_sms, cudaStream_t s);
+cudaError_t launch_lateral_pairs_256(const Plan& p, const LateralParams& lp, const void* tmap, int num_sms, cudaStream_t s);
+cudaError_t launch_lateral_pairs_512(const Plan& p, const LateralParams& lp, const void* tmap, int num_sms, cudaStream_t s);
+cudaError_t launch_lateral_pairs_1024(const Plan& p, const LateralParams& lp, const void* tmap, int num_sms, cudaStream_t s);
+cudaError_t launch_lateral_pair(const Plan& p, const LateralParams& lp, int num_sms, cudaStream_t s);
+bool lateral_pupil_supported(int nx, int ny);
+cudaError_t launch_lateral_pupil(const Plan& p, const LateralParams& lp, int num_sms, cudaStream_t s);
 // Columns per column item of the lateral kernel for a column length ny.
 int lateral_col_band(int ny);
 

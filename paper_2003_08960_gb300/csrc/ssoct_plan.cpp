@@ -328,6 +328,17 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     }
   p.stage_rows = st;
   p.small_rows = lateral_small_rows(p);
+  // The work queue for non-square frames, and for the chirp table of the
+  // aberration path, where its staging fits and the sweep is long enough to fill
+  // it; the two passes through the frame buffer otherwise.  Queue against two
+  // passes: 256 x 128 x 64 22.8 / 21.5 us, 384 x 256 x 32 29.3 / 35.1, 640 x 384 x
+  // 160 251 / 332, 1024 x 512 x 64 185 / 279, 768 x 1024 x 64 with a 301 x 401
+  // window 210 / 354; loss and gradient at 384 x 384 x 32 216 / 204, 512 x 512 x
+  // 32 270 / 283, 512 x 512 x 128 753 / 830, 1024 x 1024 x 64 1450 / 1606.
+  const bool queue_fits = lateral_smem_bytes(p) <= 226u * 1024u;
+  const long long voxels = (long long)nx * ny * nlambda;
+  p.pair_queue = generic && queue_fits && voxels >= 2500000;
+  p.pupil_queue = (flags & SSOCT_FLAG_PUPIL) && lateral_pupil_supported(nx, ny) && queue_fits && voxels >= 6000000;
   if (!generic && lateral_smem_bytes(p) > 227u * 1024u) {
     delete h;
     return SSOCT_EUNSUPPORTED;  // rescale ratio too far from 1 for the staging buffer
@@ -386,6 +397,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     put(p.off_ratio, ratio.data(), sizeof(double) * ratio.size());
   }
   p.off_ring = take(sizeof(uint16_t) * (size_t)nlambda * ny * nx);
+  // (frames without a persistent kernel of their own keep their ring in the frame buffer)
   p.off_scratch = take(generic ? 0 : sizeof(float2) * (size_t)p.slots_alloc * ny * p.wxp);
   const size_t inter_bytes = sizeof(float2) * (size_t)p.wy * p.ntx * nlambda * kTile;
   p.off_inter = take(inter_bytes);
@@ -483,7 +495,8 @@ ssoct_status ssoct_set_workspace(ssoct_plan h, void* dev_ptr, size_t bytes) {
       p.ws = nullptr;
       return cuda_fail(&p, e, "chirp table upload");
     }
-  } else if (!encode_scratch_map_at(p, ws + p.off_scratch, p.slots_alloc, p.tmap)) {
+  }
+  if (!encode_scratch_map_at(p, ws + (p.generic ? p.off_F : p.off_scratch), p.slots_alloc, p.tmap)) {
     p.ws = nullptr;
     return fail(&p, SSOCT_ECUDA, "cuTensorMapEncodeTiled failed for the scratch ring");
   }
@@ -541,7 +554,7 @@ ssoct_status ssoct_push_frames(ssoct_plan h, const uint16_t* frames, int n, int 
 // (tab0 + f) % nl.  The schedule covers all nl frames.
 static LateralParams lateral_params(const Plan& p, const uint16_t* frames, int ring_start, int tab0) {
   char* ws = p.ws;
-  LateralParams lp;
+  LateralParams lp = {};
   lp.frames = frames;
   lp.ring_start = ring_start;
   lp.tab0 = tab0;
@@ -556,7 +569,7 @@ static LateralParams lateral_params(const Plan& p, const uint16_t* frames, int r
   lp.cy2 = (const float2*)(ws + p.off_cy2);
   lp.twx = (const float2*)(ws + p.off_twx);
   lp.twy = (const float2*)(ws + p.off_twy);
-  lp.scratch = (float2*)(ws + p.off_scratch);
+  lp.scratch = (float2*)(ws + (p.generic ? p.off_F : p.off_scratch));
   lp.inter = (float2*)(ws + p.off_inter);
   lp.ctr = (Counters*)(ws + p.off_ctr);
   lp.rows_done = (unsigned*)(ws + p.off_ctr + sizeof(Counters));
@@ -574,7 +587,7 @@ static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaSt
   char* ws = p.ws;
   // the work queue's counters; paths without a queue leave the error word to ssoct_sync
   cudaError_t e = cudaSuccess;
-  if (!p.generic && !lateral_small(p))
+  if (p.pair_queue || (!p.generic && !lateral_small(p)))
     e = cudaMemsetAsync(ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
   if (p.inject_skip) {
@@ -604,7 +617,9 @@ static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaSt
     if (e != cudaSuccess) return cuda_fail(&p, e, "rescale-axial kernel launch");
     if (*ev) cudaEventRecord((*ev)[1], s);
   }
-  e = p.generic ? launch_lateral_generic(p, lp.frames, lp.ring_start, s) : launch_lateral(p, lp, s);
+  e = p.pair_queue ? launch_lateral_pair(p, lp, p.num_sms, s)
+      : p.generic  ? launch_lateral_generic(p, lp.frames, lp.ring_start, s)
+                   : launch_lateral(p, lp, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "lateral kernel launch");
   if (p.axial_first) {
     if (*ev) cudaEventRecord((*ev)[2], s);
@@ -862,7 +877,16 @@ ssoct_status ssoct_sharpness(ssoct_plan h, const uint16_t* frames_dev, float* vo
     if (e != cudaSuccess) return cuda_fail(&p, e, "pupil table kernel");
     p.sh_dirty = false;
   }
-  e = launch_sharpness(p, frames_dev, vol_dev, s);
+  const bool queue = p.pupil_queue && (uintptr_t)frames_dev % 16 == 0;  // the queue's bulk copies; any frames otherwise
+  if (queue) {
+    e = cudaMemsetAsync(p.ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
+    LateralParams lp = lateral_params(p, frames_dev, 0, 0);
+    lp.cp = (const float2*)(p.ws + p.off_cp);
+    e = launch_lateral_pupil(p, lp, p.num_sms, s);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "lateral kernel launch");
+  }
+  e = launch_sharpness(p, frames_dev, vol_dev, queue, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "sharpness kernels");
   e = cudaMemcpyAsync(out_host, p.ws + p.off_red + 2 * sizeof(double), 17 * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "loss and gradient read-back");
