@@ -345,10 +345,10 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) rescale_axial_kernel(co
 //    X(p + 32) = (Z_q - conj Z_{N-q}) / (2i);
 //  * every frame's two source rows of the tile (the rows of its y taps) are
 //    staged in shared memory by one 2D tensor copy per frame (TMA), which
-//    reads zeros outside the frame; the next tile's copies are issued as soon
-//    as the current tile's samples have been read, and land while it finishes
-//    its transform and writes its planes.  (16-byte cp.async copies of the
-//    same rows, ten per row, took 0.39 of 0.88 ms at 1024 x 1024 x 256);
+//    reads zeros outside the frame.  A warp samples frames of its own and
+//    stages them by itself, on a barrier of its own: its copies of the next
+//    tile are issued as soon as it has its samples, and land while it finishes
+//    its transform and writes its planes;
 //  * the x taps of Eq. 5 follow u(x0 + k) = u(x0) + k s_t along the strip, so
 //    one record per (frame, strip), built in float64 (first staged column,
 //    integer and fractional part of u(x0) relative to it, s_t - 1), gives every
@@ -358,9 +358,18 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) rescale_axial_kernel(co
 // The DFT over t is a two-stage split N1 x N2 (ra_split_n1: the axial
 // kernel's where that gives 8 to 16 warps per tile, 16 x 6, 16 x 10 and
 // 20 x 10 for 96, 160 and 200 frames): N2-point DFTs in registers, twiddle,
-// exchange through shared memory, N1-point DFTs (idle in some threads where N1
-// does not divide N2), the second stage in place, so that the pair separation
-// reads Z_{N-q} from the same buffer after a barrier.
+// exchange through shared memory, N1-point DFTs.  A warp of the second stage has
+// the columns k2 and N2 - k2 of 16 series in its two halves, so the pair
+// separation takes Z_{N-q} by shuffles, and the warps meet twice per tile only,
+// around the exchange.
+// Bound: 104 M instructions at 512 x 512 x 256 (49 per pixel and frame, 23 of
+// them floating point) issue in 58 % of the cycles; the rest is mostly the wait
+// for the staging copies.  Measured against copies and records staged by the CTA
+// and a third barrier around the separation: 1024 x 1024 x 256 610 -> 560 us,
+// 768 x 768 x 200 320 -> 246, 640 x 640 x 160 183 -> 141, 512 x 512 x 128 93 ->
+// 80, 384 x 384 x 96 54 -> 40, 256 x 256 x 64 21 -> 17.  Not faster: 16-byte
+// cp.async pieces (632 us), one copy per two frames (560), tiles of 32 pixels with
+// two CTAs per SM (657), one elected lane issuing the copies (598).
 struct RescaleAxialTileParams {
   int ring_start;            // gate frame t is frame (ring_start + t) mod nl of the tensor map
   const StripTap* xstrip;    // [nl][nx / 64]
@@ -376,27 +385,31 @@ struct RescaleAxialTileParams {
 
 constexpr int kRaStrip = 64;  // pixels per tile (two per complex series)
 
-// Eq. 5 at strip pixel k of a frame whose two staged source rows are r0, r1.
-__device__ __forceinline__ float ra_sample(int k, const StripTap& xs, const Tap& yt, const uint16_t* r0,
-                                           const uint16_t* r1) {
-  const float g = fmaf((float)k, xs.e, xs.f);
-  const float fl = floorf(g);
-  const float fr = g - fl;
-  const int col = xs.off + k + (int)fl;
-  const float a0 = __uint2float_rn(r0[col]), a1 = __uint2float_rn(r0[col + 1]);
-  const float b0 = __uint2float_rn(r1[col]), b1 = __uint2float_rn(r1[col + 1]);
-  const float h0 = fmaf(fr, a1 - a0, a0), h1 = fmaf(fr, b1 - b0, b0);
-  return fmaf(yt.w0, h0, yt.w1 * h1);
+// Eq. 5 at strip pixels k and k + 32 of a frame whose two staged source rows are
+// r0 and r0 + w.
+__device__ __forceinline__ float2 ra_sample(int k, const StripTap& xs, const Tap& yt, const uint16_t* r0, int w) {
+  const uint16_t* at = r0 + (xs.off + k);
+  auto one = [&](int ahead) {
+    const float g = fmaf((float)(k + ahead), xs.e, xs.f);
+    const float fl = floorf(g);
+    const float fr = g - fl;
+    const uint16_t* c = at + (int)fl + ahead;
+    const float a0 = __uint2float_rn(c[0]), a1 = __uint2float_rn(c[1]);
+    const float b0 = __uint2float_rn(c[w]), b1 = __uint2float_rn(c[w + 1]);
+    const float h0 = fmaf(fr, a1 - a0, a0), h1 = fmaf(fr, b1 - b0, b0);
+    return fmaf(yt.w0, h0, yt.w1 * h1);
+  };
+  return make_float2(one(0), one(32));
 }
 
 template <int NL>
 struct RaTile {
   static constexpr int N1 = ra_split_n1(NL), N2 = NL / N1;
-  using S2 = Stage2<NL, N1>;  // stage 2: NI N1-point DFTs per thread, idle where N1 does not divide N2
+  static_assert(N1 % 2 == 0 && N2 % 2 == 0, "mirrored bins pair up in one warp");
   static constexpr int kThreads = 32 * N1;
   // shared memory: exchange [NL][32] complex, strip records [NL], y taps [NL],
   // twiddles [NL], then frame t's two staged rows (2 x w uint16) at t * stride,
-  // then the staging mbarrier.  A tensor copy's shared-memory destination must
+  // then the warps' staging mbarriers.  A tensor copy's shared-memory destination must
   // be 128-byte aligned: the staged rows start on a 128-byte boundary and each
   // frame's block is padded to a multiple of 128 bytes.
   static constexpr size_t kStageOffset = ((size_t)NL * 32 * sizeof(float2) +
@@ -404,153 +417,177 @@ struct RaTile {
                                          128 * 128;
   static_assert(kStageOffset % 128 == 0, "staged rows on a 128-byte boundary");
   __host__ __device__ static size_t frame_stride(int w) { return ((size_t)2 * w * sizeof(uint16_t) + 127) / 128 * 128; }
-  static size_t smem_bytes(int w) { return kStageOffset + (size_t)NL * frame_stride(w) + sizeof(uint64_t); }
+  static size_t smem_bytes(int w) { return kStageOffset + (size_t)NL * frame_stride(w) + N1 * sizeof(uint64_t); }
 };
 
-template <int NL>
+// W: staged columns per source row when known at compile time (kRaWidth, what
+// sweeps of up to about 1.1 of their first wavelength need: then every offset in
+// the staging area is a constant), 0 for p.w.
+constexpr int kRaWidth = 80;
+template <int NL, int W>
 __global__ void __launch_bounds__(RaTile<NL>::kThreads, 1)
     rescale_axial_tile_kernel(const __grid_constant__ RescaleAxialTileParams p,
                               const __grid_constant__ CUtensorMap fmap) {
   using R = RaTile<NL>;
   constexpr int N1 = R::N1, N2 = R::N2, T = R::kThreads;
-  using S2 = typename R::S2;
-  static_assert(T >= NL, "one loader thread per frame");
+  static_assert(N2 <= 32, "one lane per frame of a warp");
   // its own name: the other kernels of this file declare the dynamic shared
   // memory with 16-byte alignment, and a tensor copy needs 128 here
   extern __shared__ __align__(1024) unsigned char smem_ra[];
+  __shared__ unsigned gave_up;
   unsigned char* smem = smem_ra;
   float2* ex = reinterpret_cast<float2*>(smem);
   StripTap* xsm = reinterpret_cast<StripTap*>(ex + NL * 32);
   Tap* ysm = reinterpret_cast<Tap*>(xsm + NL);
   float2* tw = reinterpret_cast<float2*>(ysm + NL);
   unsigned char* st = smem + R::kStageOffset;  // frame t's rows at st + t * fstride
-  const size_t fstride = R::frame_stride(p.w);
-  uint64_t& full = *reinterpret_cast<uint64_t*>(st + NL * fstride);
+  const int w = W ? W : p.w;
+  const int fstride = (int)R::frame_stride(w);
+  uint64_t* full = reinterpret_cast<uint64_t*>(st + (size_t)NL * fstride) + threadIdx.x / 32;  // this warp's
   const int tid = threadIdx.x;
   const int pp = tid % 32, j1 = tid / 32;
-  const int w = p.w;
   const int strips = p.nx / kRaStrip;
   const int ntiles = strips * p.ny;
   const size_t plane = (size_t)p.ny * p.nx;
   for (int i = tid; i < NL; i += T) tw[i] = p.twl[i];
-  if (tid == 0) {
-    mbar_init(&full, 1);
+  if (tid == 0) gave_up = 0u;
+  if (pp == 0) {
+    mbar_init(full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  // loader role: thread t < NL stages frame t's two source rows of a tile
-  const bool loader = tid < NL;
-  const int frow = loader ? ((p.ring_start + tid) % NL) * p.ny : 0;  // first row of frame t in the map
-  const unsigned tile_bytes = (unsigned)(NL * 2 * w * sizeof(uint16_t));
-  auto stage = [&](const StripTap& xr, const Tap& yr) {
-    if (tid == 0) mbar_arrive_tx(&full, tile_bytes);
-    if (loader) {
-      xsm[tid] = xr;
-      ysm[tid] = yr;
-      // earlier generic reads of the buffer come before this async-proxy write
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      unsigned char* dst = st + (size_t)tid * fstride;
+  // Warp j1 samples the frames t = j1 + N1 j2 and is the only one to read their
+  // staged rows and records, so it refills them by itself: lane j2 < N2 stages
+  // frame t's two source rows of the next tile as soon as the warp has its samples.
+  const int t_own = j1 + N1 * pp;
+  const bool loader = pp < N2;
+  const int frow = loader ? ((p.ring_start + t_own) % NL) * p.ny : 0;  // first row of the frame in the map
+  // lanes l0 .. l1 - 1 stage their frames (l0 = 0 opens the barrier's phase for all)
+  auto stage = [&](int l0, int l1, const StripTap& xr, const Tap& yr) {
+    if (l0 == 0 && pp == 0) mbar_arrive_tx(full, (unsigned)(N2 * 2 * w * sizeof(uint16_t)));
+    __syncwarp();
+    if (pp >= l0 && pp < l1) {
+      xsm[t_own] = xr;
+      ysm[t_own] = yr;
+      unsigned char* dst = st + (size_t)t_own * fstride;
       // a tensor copy needs a 128-byte aligned destination and an x start whose
       // byte offset is a multiple of 16; a copy that would break either is not
       // issued (the wait for it then runs out and reports kErrAxial)
       if ((smem_u32(dst) & 127u) == 0u && (xr.xs & 7) == 0)
-        tma_load_2d(dst, &fmap, xr.xs, frow + yr.base, &full);
+        tma_load_2d(dst, &fmap, xr.xs, frow + yr.base, full);
       else
         atomicOr(p.err, kErrAxial);
     }
+    __syncwarp();
   };
   auto records = [&](int tile, StripTap& xr, Tap& yr) {
     if (loader && tile < ntiles) {
       const int y = tile / strips, strip = tile - y * strips;
-      xr = p.xstrip[(size_t)tid * strips + strip];
-      yr = p.ytab[(size_t)tid * p.ny + y];
+      xr = p.xstrip[(size_t)t_own * strips + strip];
+      yr = p.ytab[(size_t)t_own * p.ny + y];
     }
   };
   StripTap xr{};
   Tap yr{};
   int tile = blockIdx.x;
   unsigned phase = 0;     // tiles staged and consumed so far
-  bool pending = false;   // a staging copy is in flight on `full`
+  bool pending = false;   // this warp's staging copies are in flight
   records(tile, xr, yr);
   if (tile < ntiles) {
-    stage(xr, yr);
+    stage(0, N2, xr, yr);
     pending = true;
   }
   for (; tile < ntiles; tile += gridDim.x) {
     const int next = tile + gridDim.x;
-    records(next, xr, yr);  // in flight while this tile is transformed
-    // one thread waits for the copies; the others sleep at the barrier
-    bool ok = true;
-    if (tid == 0) {
-      ok = mbar_wait_bounded(&full, phase & 1u, kAxWaitNs);
-      if (!ok) atomicOr(p.err, kErrAxial);
+    records(next, xr, yr);  // in flight while this tile is sampled
+    // the warps meet only around the exchange below
+    if (!mbar_wait_bounded(full, phase & 1u, kAxWaitNs)) {
+      atomicOr(p.err, kErrAxial);
+      gave_up = 1u;
+    } else {
+      pending = false;
+      ++phase;
     }
-    // this tile's rows and records are in; every thread is done with the last tile
-    if (__syncthreads_or(!ok)) break;
-    pending = false;
-    ++phase;
     const int y = tile / strips, strip = tile - y * strips;
     // 1. Eq. 5 samples of frames t = j1 + N1 j2 at pixels pp and pp + 32 (one
-    //    complex series), N2-point DFT over j2, twiddle, exchange
-    float2 a[S2::A];
+    //    complex series), N2-point DFT over j2, twiddle
+    float2 a[N1 > N2 ? N1 : N2];
+    // the chirp at this lane's pixels of step 2, requested here
+    const int s = (j1 & 1) * 16 + (pp & 15);
+    const int xa = strip * kRaStrip + s;
+    const float2 cyv = ldg2(p.cy + y), cxa = ldg2(p.cx + xa), cxb = ldg2(p.cx + xa + 32);
+    const unsigned char* rows = st + j1 * fstride;
+    // With 256 frames the copies of the first half of a warp's frames are issued
+    // before it samples the second half (578 -> 560 us at 1024 x 1024; in quarters
+    // 576).  Fewer frames are slower so (80 -> 84 at 512 x 512 x 128, 246 -> 257 at
+    // 768 x 768 x 200): their warps find the copies done anyway.
+    constexpr int kRaParts = NL == 256 ? 2 : 1;
+    constexpr int kRefill = (N2 + kRaParts - 1) / kRaParts;
+    const bool refill = !pending && next < ntiles;
+    static_for<0, kRaParts>([&](auto G) {
+      constexpr int lo = decltype(G)::value * kRefill, hi = lo + kRefill < N2 ? lo + kRefill : N2;
 #pragma unroll
-    for (int j2 = 0; j2 < N2; ++j2) {
-      const int t = j1 + N1 * j2;
-      const StripTap xs = xsm[t];
-      const Tap yt = ysm[t];
-      const uint16_t* r0 = reinterpret_cast<const uint16_t*>(st + (size_t)t * fstride);
-      a[j2] = make_float2(ra_sample(pp, xs, yt, r0, r0 + w), ra_sample(pp + 32, xs, yt, r0, r0 + w));
-    }
-    Dft<N2, -1>::template run<1, 0>(a);
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * 32 + pp] = cmul(a[k2], tw[k2 * N1 + j1]);
-    __syncthreads();  // the staged rows are read: the next tile's copies may overwrite them
-    if (next < ntiles) {
-      stage(xr, yr);
-      pending = true;
-    }
-    // 2. N1-point DFTs, results back into the slots just read: Z_q, q = k2 + N2 k1,
-    //    at row k2 N1 + k1
-    static_for<0, S2::NI>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      const int k2 = j1 + N1 * i;
-      if (!S2::live(i, j1)) return;
-#pragma unroll
-      for (int jj = 0; jj < N1; ++jj) a[i * N1 + jj] = ex[(k2 * N1 + jj) * 32 + pp];
-      Dft<N1, -1>::template run<1, i * N1>(a);
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) ex[(k2 * N1 + k1) * 32 + pp] = a[i * N1 + k1];
-    });
-    __syncthreads();
-    // 3. the two real series' spectra, bins q = 0 .. NL/2, as plane rows, times
-    //    the input chirp and |K| of Eq. 6 at their pixels (the factor 1/2 of the
-    //    separation folded in)
-    const int xa = strip * kRaStrip + pp;
-    float2* dst = p.planes + (size_t)y * p.nx + xa;
-    const float2 cyv = ldg2(p.cy + y);
-    const float h = 0.5f * p.k_abs;
-    float2 ca = cmul(ldg2(p.cx + xa), cyv), cb = cmul(ldg2(p.cx + xa + 32), cyv);
-    ca = make_float2(ca.x * h, ca.y * h);
-    cb = make_float2(cb.x * h, cb.y * h);
-    static_for<0, S2::NI>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      const int k2 = j1 + N1 * i;
-      if (!S2::live(i, j1)) return;
-#pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) {
-        const int q = k2 + N2 * k1;
-        if (q <= NL / 2) {
-          const int qm = (NL - q) % NL;
-          const float2 zq = a[i * N1 + k1];
-          const float2 zm = ex[((qm % N2) * N1 + qm / N2) * 32 + pp];
-          __stcs(dst + (size_t)q * plane, cmul(make_float2(zq.x + zm.x, zq.y - zm.y), ca));
-          __stcs(dst + (size_t)q * plane + 32, cmul(make_float2(zq.y + zm.y, zm.x - zq.x), cb));
-        }
+      for (int j2 = lo; j2 < hi; ++j2) {
+        const int t = j1 + N1 * j2;
+        a[j2] = ra_sample(pp, xsm[t], ysm[t], reinterpret_cast<const uint16_t*>(rows + j2 * (N1 * fstride)), w);
+      }
+      if (refill && lo < hi) {
+        // the lanes' reads of the rows come before the async-proxy writes
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        stage(lo, hi, xr, yr);
+        pending = true;
       }
     });
+    Dft<N2, -1>::template run<1, 0>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) a[k2] = cmul(a[k2], tw[k2 * N1 + j1]);
+    __syncthreads();  // every warp has read the last tile's exchange
+    if (gave_up) break;
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) ex[(k2 * N1 + j1) * 32 + pp] = a[k2];
+    __syncthreads();  // the exchange is written
+    // 2. N1-point DFTs, Z_q for q = k2 + N2 k1, and the two real series' spectra
+    //    from Z_q and Z_{N-q} = Z at (N2 - k2, N1 - 1 - k1).  A warp takes 16
+    //    series of the two columns k2 = c and N2 - c, one in each half, so that
+    //    the mirrored values come from lane ^ 16 and no warp waits for another;
+    //    columns 0 and N2 / 2 mirror into themselves.
+    const float h = 0.5f * p.k_abs;  // the factor 1/2 of the separation folded in
+    for (int u = j1; u < N2; u += N1) {  // N1 is even: every unit of a warp has its half s
+      const int c = u / 2;
+      const bool upper = pp >= 16;
+      const int k2 = c == 0 ? (upper ? N2 / 2 : 0) : (upper ? N2 - c : c);
+#pragma unroll
+      for (int jj = 0; jj < N1; ++jj) a[jj] = ex[(k2 * N1 + jj) * 32 + s];
+      Dft<N1, -1>::template run<1, 0>(a);
+      float2 ca = cmul(cxa, cyv), cb = cmul(cxb, cyv);
+      ca = make_float2(ca.x * h, ca.y * h);
+      cb = make_float2(cb.x * h, cb.y * h);
+      float2* dst = p.planes + ((size_t)k2 * p.ny + y) * p.nx + xa;
+      // plane rows of bin k2 + N2 k1, times the input chirp and |K| of Eq. 6
+      auto put = [&](int k1, float2 zq, float2 zm) {
+        float2* d = dst + (size_t)(N2 * k1) * plane;
+        __stcs(d, cmul(make_float2(zq.x + zm.x, zq.y - zm.y), ca));
+        __stcs(d + 32, cmul(make_float2(zq.y + zm.y, zm.x - zq.x), cb));
+      };
+      if (c != 0) {
+#pragma unroll
+        for (int k1 = 0; k1 < N1 / 2; ++k1) {
+          const float2 o = a[N1 - 1 - k1];
+          const float2 zm = make_float2(__shfl_xor_sync(0xffffffffu, o.x, 16), __shfl_xor_sync(0xffffffffu, o.y, 16));
+          put(k1, a[k1], zm);
+        }
+      } else if (upper) {
+#pragma unroll
+        for (int k1 = 0; k1 < N1 / 2; ++k1) put(k1, a[k1], a[N1 - 1 - k1]);
+      } else {
+#pragma unroll
+        for (int k1 = 0; k1 <= N1 / 2; ++k1) put(k1, a[k1], a[(N1 - k1) % N1]);
+      }
+    }
   }
-  // after a time-out, the copy still in flight lands before the CTA exits
-  if (pending && tid == 0 && !mbar_wait_bounded(&full, phase & 1u, kAxWaitNs)) atomicOr(p.err, kErrAxial);
+  // after a time-out, the copies still in flight land before the CTA exits
+  if (pending && !mbar_wait_bounded(full, phase & 1u, kAxWaitNs)) atomicOr(p.err, kErrAxial);
 }
 
 struct GateCutsParams {
@@ -746,13 +783,13 @@ template <int NL>
 cudaError_t launch_ra_tiles(const RescaleAxialTileParams& rp, const CUtensorMap& fmap, int num_sms, cudaStream_t s) {
   using R = RaTile<NL>;
   const size_t smem = R::smem_bytes(rp.w);
-  cudaError_t e = cudaFuncSetAttribute(rescale_axial_tile_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  const auto kernel = rp.w == kRaWidth ? rescale_axial_tile_kernel<NL, kRaWidth> : rescale_axial_tile_kernel<NL, 0>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long ntiles = (long long)(rp.nx / kRaStrip) * rp.ny;
   long long grid = num_sms > 0 ? num_sms : 1;
   if (grid > ntiles) grid = ntiles;
-  rescale_axial_tile_kernel<NL><<<(unsigned)grid, R::kThreads, smem, s>>>(rp, fmap);
+  kernel<<<(unsigned)grid, R::kThreads, smem, s>>>(rp, fmap);
   return cudaGetLastError();
 }
 
