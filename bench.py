@@ -231,7 +231,9 @@ def run_ssoct(args):
         os.unlink(tune_cache)  # the tuner writes it; other plans of the bench read the choice back
         tune = plan.autotune(frames, tune_cache, stream)
     tc_main = args.tc_axial or bool(tune and tune["tc_axial"])
-    af_main = args.axial_first or bool(tune and tune["axial_first"])
+    # untuned plans of these frames run axial-first where the sweep offers it
+    af_main = args.axial_first or bool(tune["axial_first"] if tune else
+                                       not args.tc_axial and w.nx == w.ny and w.nx >= 256 and w.nlambda in (64, 96, 128, 160, 200, 256))
     xy = torch.empty((wy, wx), dtype=torch.float32, device="cuda")
     xz = torch.empty((nl, wx), dtype=torch.float32, device="cuda")
     yz = torch.empty((nl, wy), dtype=torch.float32, device="cuda")

@@ -78,7 +78,11 @@ typedef enum {
  * directly.  Eq. 6 is linear and identical for every frame, so V is the same as
  * in the paper's order; HBM traffic drops from 22 to 14 B per voxel.  Frame
  * sizes of the persistent lateral kernel and even nlambda only; no sliding
- * gates, no no-allocation call, not with SSOCT_FLAG_TC_AXIAL (EUNSUPPORTED). */
+ * gates, no no-allocation call, not with SSOCT_FLAG_TC_AXIAL (EUNSUPPORTED).
+ * Plans made without the flag run whole volumes in this order too where it is
+ * the faster one and they offer it (see ssoct_autotune): square frames of 256 and
+ * more with a window of at least 7/8 of the plane; their sliding gates and
+ * no-allocation calls keep the paper's order. */
 #define SSOCT_FLAG_AXIAL_FIRST 0x8u
 
 /* Read-only facts about a plan. */
