@@ -74,44 +74,44 @@ def ssoct_workspace_bytes(plan):
 
 
 def ssoct_set_workspace(plan, dev_ptr: int, nbytes: int) -> int:
-    return _abi.lib().ssoct_set_workspace(plan, C.c_void_p(dev_ptr), nbytes)
+    return _abi.lib().ssoct_set_workspace(plan, dev_ptr, nbytes)
 
 
 def ssoct_push_frames(plan, frames_ptr: int, n: int, frames_on_device: bool, first_seq: int, stream: int) -> int:
-    return _abi.lib().ssoct_push_frames(plan, C.c_void_p(frames_ptr), n, int(bool(frames_on_device)),
-                                        first_seq, C.c_void_p(stream))
+    return _abi.lib().ssoct_push_frames(plan, frames_ptr, n, int(bool(frames_on_device)),
+                                        first_seq, stream)
 
 
 def ssoct_reconstruct_volume(plan, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_volume(plan, C.c_void_p(vol_ptr), C.c_void_p(complex_ptr or None),
-                                               C.c_void_p(stream))
+    return _abi.lib().ssoct_reconstruct_volume(plan, vol_ptr, complex_ptr or None,
+                                               stream)
 
 
 def ssoct_reconstruct_frames(plan, frames_ptr: int, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_frames(plan, C.c_void_p(frames_ptr), C.c_void_p(vol_ptr),
-                                               C.c_void_p(complex_ptr or None), C.c_void_p(stream))
+    return _abi.lib().ssoct_reconstruct_frames(plan, frames_ptr, vol_ptr,
+                                               complex_ptr or None, stream)
 
 
 def ssoct_reconstruct_sliding(plan, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_sliding(plan, C.c_void_p(vol_ptr), C.c_void_p(complex_ptr or None),
-                                                C.c_void_p(stream))
+    return _abi.lib().ssoct_reconstruct_sliding(plan, vol_ptr, complex_ptr or None,
+                                                stream)
 
 
 def ssoct_reconstruct_frames_noalloc(plan, frames_ptr: int, vol_ptr: int, complex_ptr: int, stream: int) -> int:
     """ssoct_reconstruct_frames without any device allocation (scratch in a fixed
     64 MiB device array inside the library); the plan needs no workspace."""
-    return _abi.lib().ssoct_reconstruct_frames_noalloc(plan, C.c_void_p(frames_ptr), C.c_void_p(vol_ptr),
-                                                       C.c_void_p(complex_ptr or None), C.c_void_p(stream))
+    return _abi.lib().ssoct_reconstruct_frames_noalloc(plan, frames_ptr, vol_ptr,
+                                                       complex_ptr or None, stream)
 
 
 def ssoct_get_cuts(plan, vol_ptr: int, x0: int, y0: int, z0: int, xy_ptr: int, xz_ptr: int, yz_ptr: int,
                    stream: int) -> int:
-    return _abi.lib().ssoct_get_cuts(plan, C.c_void_p(vol_ptr), x0, y0, z0, C.c_void_p(xy_ptr or None),
-                                     C.c_void_p(xz_ptr or None), C.c_void_p(yz_ptr or None), C.c_void_p(stream))
+    return _abi.lib().ssoct_get_cuts(plan, vol_ptr, x0, y0, z0, xy_ptr or None,
+                                     xz_ptr or None, yz_ptr or None, stream)
 
 
 def ssoct_sync(plan, stream: int) -> int:
-    return _abi.lib().ssoct_sync(plan, C.c_void_p(stream))
+    return _abi.lib().ssoct_sync(plan, stream)
 
 
 def ssoct_set_pupil(plan, coeffs: Sequence[float], z_m: float) -> int:
@@ -122,14 +122,14 @@ def ssoct_set_pupil(plan, coeffs: Sequence[float], z_m: float) -> int:
 def ssoct_sharpness(plan, frames_ptr: int, vol_ptr: int, stream: int):
     """Returns (status, out[17]): loss, dL/dz, dL/dc_1 .. dL/dc_15."""
     out = np.zeros(17, dtype=np.float64)
-    st = _abi.lib().ssoct_sharpness(plan, C.c_void_p(frames_ptr), C.c_void_p(vol_ptr),
-                                    out.ctypes.data_as(C.POINTER(C.c_double)), C.c_void_p(stream))
+    st = _abi.lib().ssoct_sharpness(plan, frames_ptr, vol_ptr,
+                                    out.ctypes.data_as(C.POINTER(C.c_double)), stream)
     return st, out
 
 
 def ssoct_sliding_cuts(plan, x0: int, y0: int, z0: int, xy_ptr: int, xz_ptr: int, yz_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_sliding_cuts(plan, x0, y0, z0, C.c_void_p(xy_ptr or None), C.c_void_p(xz_ptr or None),
-                                         C.c_void_p(yz_ptr or None), C.c_void_p(stream))
+    return _abi.lib().ssoct_sliding_cuts(plan, x0, y0, z0, xy_ptr or None, xz_ptr or None,
+                                         yz_ptr or None, stream)
 
 
 def ssoct_inject_stall(plan, skip: int, wait_limit_ns: int) -> int:
@@ -163,17 +163,24 @@ def ssoct_destroy_plan(plan) -> None:
 
 # ---------------------------------------------------------------- convenience
 
+_torch_with_gpu = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("libssoct needs a CUDA device; there is no CPU path")
-    return torch
+    global _torch_with_gpu
+    if _torch_with_gpu is None:  # asked until a device is there, then remembered
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("libssoct needs a CUDA device; there is no CPU path")
+        _torch_with_gpu = torch
+    return _torch_with_gpu
 
 
 def _stream_ptr(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Plan:
