@@ -23,6 +23,7 @@ namespace {
 
 template <int NL>
 __global__ void __launch_bounds__(kTile * Split<NL>::N1) axial_kernel(const __grid_constant__ AxialParams p) {
+  after_previous_kernel();
   constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
   static_assert(N2 % N1 == 0, "the second stage needs N1 | N2");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -184,6 +185,7 @@ __device__ __forceinline__ void axial_epilogue(const AxialParams& p, const float
 template <int NL>
 __global__ void __launch_bounds__(AxStream<NL>::kThreadsAll, 1)
     axial_stream_kernel(const __grid_constant__ AxialParams p, const __grid_constant__ CUtensorMap imap) {
+  after_previous_kernel();
   using S = AxStream<NL>;
   using S2 = typename S::S2;
   constexpr int N1 = S::N1, N2 = S::N2, T = S::kGroupThreads, P = S::kPix;
@@ -289,6 +291,7 @@ struct RescaleAxialParams {
 // lateral pass's DFTs as they are, and the mirrored bins take c^2 there.
 template <int NL>
 __global__ void __launch_bounds__(kTile * Split<NL>::N1) rescale_axial_kernel(const __grid_constant__ RescaleAxialParams p) {
+  after_previous_kernel();
   constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
   static_assert(N2 % N1 == 0, "the second stage needs N1 | N2");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -428,6 +431,7 @@ template <int NL, int W>
 __global__ void __launch_bounds__(RaTile<NL>::kThreads, 1)
     rescale_axial_tile_kernel(const __grid_constant__ RescaleAxialTileParams p,
                               const __grid_constant__ CUtensorMap fmap) {
+  after_previous_kernel();
   using R = RaTile<NL>;
   constexpr int N1 = R::N1, N2 = R::N2, T = R::kThreads;
   static_assert(N2 <= 32, "one lane per frame of a warp");
@@ -611,6 +615,7 @@ __device__ __forceinline__ float envelope(float2 v, float scale, int magnitude) 
 // xy cut at depth bin z0 straight from the intermediate: at every window pixel
 // the single bin V_z0 = sum_t H_t exp(-2 pi i z0 t / N) of Eq. 7.
 __global__ void __launch_bounds__(256) gate_xy_kernel(const __grid_constant__ GateCutsParams c) {
+  after_previous_kernel();
   extern __shared__ __align__(16) unsigned char smem[];
   float2* w = reinterpret_cast<float2*>(smem);
   for (int k = threadIdx.x; k < c.nl; k += blockDim.x) w[k] = ldg2(c.wq + k);
@@ -661,6 +666,7 @@ struct XySlideParams {
 constexpr int kSlideAhead = 8;
 
 __global__ void __launch_bounds__(256) xy_slide_kernel(const __grid_constant__ XySlideParams c) {
+  after_previous_kernel();
   extern __shared__ __align__(16) unsigned char smem[];
   float2* w = reinterpret_cast<float2*>(smem);  // the slots' factors exp(-2 pi i z0 t / nl), in the order they are read
   for (int j = threadIdx.x; j < c.k; j += blockDim.x) w[j] = ldg2(c.wq + (int)((long long)c.z0 * ((c.slot0 + j) % c.nl) % c.nl));
@@ -714,6 +720,7 @@ constexpr int kLinePix = 8;
 
 template <int NL>
 __global__ void __launch_bounds__(kLinePix * ax_split_n1(NL)) gate_lines_kernel(const __grid_constant__ GateCutsParams c) {
+  after_previous_kernel();
   constexpr int N1 = ax_split_n1(NL), N2 = NL / N1, P = kLinePix;
   using S2 = Stage2<NL, N1>;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -763,11 +770,11 @@ __global__ void __launch_bounds__(kLinePix * ax_split_n1(NL)) gate_lines_kernel(
 }
 
 template <int NL>
-cudaError_t launch_lines(const GateCutsParams& c, cudaStream_t s) {
+cudaError_t launch_lines(const GateCutsParams& c, bool late, cudaStream_t s) {
   const size_t smem = (size_t)NL * kLinePix * sizeof(float2);  // at most 32 KB
   const int blocks = (c.xz ? (c.wx + kLinePix - 1) / kLinePix : 0) + (c.yz ? (c.wy + kLinePix - 1) / kLinePix : 0);
-  gate_lines_kernel<NL><<<blocks, kLinePix * ax_split_n1(NL), smem, s>>>(c);
-  return cudaGetLastError();
+  return late ? launch_after(gate_lines_kernel<NL>, dim3(blocks), kLinePix * ax_split_n1(NL), smem, s, c)
+              : launch_next(gate_lines_kernel<NL>, dim3(blocks), kLinePix * ax_split_n1(NL), smem, s, c);
 }
 
 template <int NL>
@@ -775,8 +782,7 @@ cudaError_t launch_ra(const RescaleAxialParams& rp, cudaStream_t s) {
   const size_t smem = (size_t)NL * kTile * sizeof(float2);
   cudaError_t e = cudaFuncSetAttribute(rescale_axial_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  rescale_axial_kernel<NL><<<dim3(rp.nx / kTile, rp.ny), kTile * Split<NL>::N1, smem, s>>>(rp);
-  return cudaGetLastError();
+  return launch_next(rescale_axial_kernel<NL>, dim3(rp.nx / kTile, rp.ny), kTile * Split<NL>::N1, smem, s, rp);
 }
 
 template <int NL>
@@ -789,8 +795,7 @@ cudaError_t launch_ra_tiles(const RescaleAxialTileParams& rp, const CUtensorMap&
   const long long ntiles = (long long)(rp.nx / kRaStrip) * rp.ny;
   long long grid = num_sms > 0 ? num_sms : 1;
   if (grid > ntiles) grid = ntiles;
-  kernel<<<(unsigned)grid, R::kThreads, smem, s>>>(rp, fmap);
-  return cudaGetLastError();
+  return launch_next(kernel, dim3((unsigned)grid), R::kThreads, smem, s, rp, fmap);
 }
 
 template <int NL>
@@ -810,8 +815,8 @@ cudaError_t launch_stream(const AxialParams& ap, int num_sms, cudaStream_t s) {
   long long grid = (long long)(num_sms > 0 ? num_sms : 1) * per_sm;
   if (grid > nunits) grid = nunits;
   if (grid < 1) return cudaSuccess;
-  axial_stream_kernel<NL><<<(unsigned)grid, S::kThreadsAll, smem, s>>>(ap, imap);
-  return cudaGetLastError();
+  return ap.late ? launch_after(axial_stream_kernel<NL>, dim3((unsigned)grid), S::kThreadsAll, smem, s, ap, imap)
+                 : launch_next(axial_stream_kernel<NL>, dim3((unsigned)grid), S::kThreadsAll, smem, s, ap, imap);
 }
 
 template <int NL>
@@ -823,8 +828,8 @@ cudaError_t launch(const AxialParams& ap, int num_sms, cudaStream_t s) {
   } else {
     const size_t smem = (size_t)NL * kTile * sizeof(float2);  // at most 8 KB
     dim3 grid(ap.ntx, ap.wy);
-    axial_kernel<NL><<<grid, kTile * Split<NL>::N1, smem, s>>>(ap);
-    return cudaGetLastError();
+    return ap.late ? launch_after(axial_kernel<NL>, grid, kTile * Split<NL>::N1, smem, s, ap)
+                   : launch_next(axial_kernel<NL>, grid, kTile * Split<NL>::N1, smem, s, ap);
   }
 }
 
@@ -844,8 +849,10 @@ cudaError_t launch_xy_slide(const Plan& p, int slot0, int k, int z0, float sign,
   c.power_scale = (float)(p.alpha * p.alpha);
   c.magnitude = (p.flags & SSOCT_FLAG_MAGNITUDE) ? 1 : 0;
   const size_t pairs = (size_t)p.wy * p.ntx * (kTile / 2);
-  xy_slide_kernel<<<(unsigned)((pairs + 255) / 256), 256, (size_t)std::max(k, 1) * sizeof(float2), s>>>(c);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)((pairs + 255) / 256));
+  const size_t smem = (size_t)std::max(k, 1) * sizeof(float2);
+  return gate_late(p) ? launch_after(xy_slide_kernel, grid, 256, smem, s, c)
+                      : launch_next(xy_slide_kernel, grid, 256, smem, s, c);
 }
 
 cudaError_t launch_gate_cuts(const Plan& p, int x0, int y0, int z0, float* xy, float* xz, float* yz,
@@ -864,11 +871,12 @@ cudaError_t launch_gate_cuts(const Plan& p, int x0, int y0, int z0, float* xy, f
   c.magnitude = (p.flags & SSOCT_FLAG_MAGNITUDE) ? 1 : 0;
   cudaError_t e = cudaSuccess;
   if (xy) {
-    gate_xy_kernel<<<4 * p.num_sms, 256, (size_t)p.nl * sizeof(float2), s>>>(c);
-    e = cudaGetLastError();
+    const size_t smem = (size_t)p.nl * sizeof(float2);
+    e = gate_late(p) ? launch_after(gate_xy_kernel, dim3(4 * p.num_sms), 256, smem, s, c)
+                     : launch_next(gate_xy_kernel, dim3(4 * p.num_sms), 256, smem, s, c);
   }
   if (e != cudaSuccess || (!xz && !yz)) return e;
-#define X(a) if (p.nl == a) return launch_lines<a>(c, s);
+#define X(a) if (p.nl == a) return launch_lines<a>(c, gate_late(p), s);
   SSOCT_AXIAL_SIZES(X)
 #undef X
   return cudaErrorInvalidValue;
@@ -951,8 +959,29 @@ cudaError_t launch_axial(const Plan& p, const AxialParams& ap, cudaStream_t s) {
   return launch_axial_with(p, ap, p.num_sms, s);
 }
 
+// Frames from the caller's device memory into the ring: 16-byte pieces, four a
+// thread in flight.  A kernel of the call's own chain: a device-to-device
+// cudaMemcpyAsync of 13 frames of 1024 x 1024 cost about 35 us between kernels.
+__global__ void __launch_bounds__(256) copy_frames_kernel(uint4* dst, const uint4* src, size_t n) {
+  after_previous_kernel();
+  const size_t first = (size_t)blockIdx.x * 1024 + threadIdx.x;
+  uint4 v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (first + 256 * k < n) v[k] = __ldcs(src + first + 256 * k);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (first + 256 * k < n) dst[first + 256 * k] = v[k];
+}
+
+cudaError_t launch_copy_frames(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  const size_t n = bytes / 16;
+  return launch_next(copy_frames_kernel, dim3((unsigned)((n + 1023) / 1024)), 256, 0, s, (uint4*)dst, (const uint4*)src, n);
+}
+
 // The three orthogonal cuts: plain gathers from the volume [q][y][x].
 __global__ void cuts_kernel(const __grid_constant__ CutsParams c) {
+  after_previous_kernel();
   const size_t nxy = c.xy ? (size_t)c.wy * c.wx : 0;
   const size_t nxz = c.xz ? (size_t)c.nl * c.wx : 0;
   const size_t nyz = c.yz ? (size_t)c.nl * c.wy : 0;
@@ -979,8 +1008,7 @@ cudaError_t launch_cuts(const CutsParams& cp, cudaStream_t s) {
   int blocks = (int)((n + 255) / 256);
   if (blocks > 1024) blocks = 1024;
   if (blocks < 1) blocks = 1;
-  cuts_kernel<<<blocks, 256, 0, s>>>(cp);
-  return cudaGetLastError();
+  return launch_next(cuts_kernel, dim3(blocks), 256, 0, s, cp);
 }
 
 }  // namespace ssoct

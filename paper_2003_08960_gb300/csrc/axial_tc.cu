@@ -237,6 +237,7 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const float (&v)[
 
 __global__ void __launch_bounds__(kTcThreads, 1)
     axial_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap imap) {
+  after_previous_kernel();
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* ring = smem;                                                      // [6][32 KB]
   unsigned short* Bs = reinterpret_cast<unsigned short*>(ring + kTcStages * kTcItemBytes);  // [hi / lo][32 x 32]
@@ -497,8 +498,8 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
   long long grid = num_sms > 0 ? num_sms : 1;  // persistent: one CTA per SM
   if (grid > nitems) grid = nitems;
   if (grid < 1) return cudaSuccess;
-  axial_tc_kernel<<<(unsigned)grid, kTcThreads, smem, s>>>(p, imap);
-  return cudaGetLastError();
+  return ap.late ? launch_after(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap)
+                 : launch_next(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap);
 }
 
 }  // namespace ssoct

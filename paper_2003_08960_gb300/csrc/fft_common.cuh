@@ -70,6 +70,45 @@ __device__ __forceinline__ void st_cg_hint(float2* a, float2 v, unsigned long lo
                : "memory");
 }
 
+// First statement of every kernel that launch_next starts: waits until the
+// kernel before it in the stream is complete and its writes are visible, then
+// lets the next one's CTAs be placed (they wait here in turn).  A kernel's
+// lifetime so begins before its predecessor's end: what another kernel of the
+// call wrote is not read with non-coherent loads (__ldg, ldg2).
+__device__ __forceinline__ void after_previous_kernel() {
+  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch that may be placed on the GPU while the kernel before it in the stream
+// drains (programmatic stream serialisation): the launch latency and the start
+// of the CTAs, 2 to 4 us between two kernels of a call, overlap its last CTAs.
+// launch_after: an ordinary launch of such a kernel.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                                const A&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                               const A&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // Eq. 5 at one pixel of a uint16 frame [.][nx] from its separable taps (weights
 // are 0 where a tap falls outside the frame; bases are clamped inside it).
 __device__ __forceinline__ float rescale_tap_value(const uint16_t* fr, int nx, const Tap& tx, const Tap& ty) {

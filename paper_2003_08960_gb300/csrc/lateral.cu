@@ -68,6 +68,7 @@ __device__ __forceinline__ float2 ld_cluster(unsigned a) {
 template <int NX, int NY, int C, bool AF>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(SmallLat<NX, NY, C>::kThreadsAll, C > 1 ? 2 : 1)
     lateral_small_kernel(const __grid_constant__ LateralParams p) {
+  after_previous_kernel();
   using L = SmallLat<NX, NY, C>;
   constexpr int T = L::kThreadsAll, PITCH = L::kPitch, RB = L::kRows;
   constexpr int N1x = Split<NX>::N1, N2x = Split<NX>::N2, N1y = Split<NY>::N1, N2y = Split<NY>::N2;
@@ -245,8 +246,7 @@ cudaError_t launch_small(const Plan& p, const LateralParams& lp, cudaStream_t s)
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  kernel<<<lp.sch.nl * C, L::kThreadsAll, smem, s>>>(lp);
-  return cudaGetLastError();
+  return launch_next(kernel, dim3(lp.sch.nl * C), L::kThreadsAll, smem, s, lp);
 }
 
 }  // namespace

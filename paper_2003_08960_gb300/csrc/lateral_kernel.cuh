@@ -188,7 +188,7 @@ __device__ __forceinline__ void row_item(const LateralParams& p, const Desc& d, 
       const float v0 = fmaf(t.w0, u16_to_f(r0[t.base]), t.w1 * u16_to_f(r0[t.base + 1]));
       const float v1 = fmaf(t.w0, u16_to_f(r1[t.base]), t.w1 * u16_to_f(r1[t.base + 1]));
       const float v = fmaf(ty.w0, v0, ty.w1 * v1);
-      const float2 c = PUP ? ldg2(cp + n) : cxs[n];
+      const float2 c = PUP ? cp[n] : cxs[n];
       a[j2] = make_float2(v * c.x, v * c.y);
     }
   }
@@ -601,6 +601,7 @@ __device__ void publisher(const LateralParams& p, uint64_t* done_bar, Handover* 
 template <int NX, int NY, bool FW, bool AF, bool PUP>
 __global__ void __launch_bounds__(kCtaThreads, 1)
     lateral_kernel(const __grid_constant__ LateralParams p, const __grid_constant__ CUtensorMap tmap) {
+  after_previous_kernel();
   static_assert(kThreads / Split<NX>::N1 <= NY, "a row item must not exceed the frame");
   static_assert(NY % band_box_rows(NY) == 0, "whole tensor copies cover a column band");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -696,8 +697,7 @@ cudaError_t launch_fw(const Plan& p, const LateralParams& lp_in, const void* tma
   if (per_sm < 1) per_sm = 1;
   int grid = (num_sms > 0 ? num_sms : 1) * per_sm;
   if (grid > total) grid = (int)total;
-  kernel<<<grid, kCtaThreads, smem, s>>>(lp, *reinterpret_cast<const CUtensorMap*>(tmap));
-  return cudaGetLastError();
+  return launch_next(kernel, grid, kCtaThreads, smem, s, lp, *reinterpret_cast<const CUtensorMap*>(tmap));
 }
 
 // Every form of a frame size: either order, with and without window bounds checks.

@@ -184,7 +184,7 @@ extern "C" ssoct_status ssoct_reconstruct_frames_noalloc(ssoct_plan h, const uin
   e = launch_lateral_with(p, lp, tmap, num_sms, s);
   if (e != cudaSuccess) return fail(p, SSOCT_ECUDA, std::string("lateral kernel launch: ") + cudaGetErrorString(e));
 
-  AxialParams ap;
+  AxialParams ap = {};
   ap.inter = lp.inter;
   ap.vol = vol_dev;
   ap.cplx = (float2*)complex_dev;

@@ -128,6 +128,7 @@ struct ShParams {
 
 template <int NX>
 __global__ void __launch_bounds__(kRowThreads) rows_fwd_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
   constexpr int N1 = Lat<NX>::N1, N2 = Lat<NX>::N2, RPI = kRowThreads / N1;
   extern __shared__ __align__(16) unsigned char smem[];
   const int r = threadIdx.x / N1, j1 = threadIdx.x % N1;
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(kRowThreads) rows_fwd_kernel(const __grid_cons
   for (int j2 = 0; j2 < N2; ++j2) {
     const int n = j1 + N1 * j2;
     const float u = rescale_tap_value(fr, NX, p.xtab[(size_t)t * NX + n], ty);
-    const float2 c = ldg2(cp + n);
+    const float2 c = cp[n];
     a[j2] = make_float2(u * c.x, u * c.y);
   }
   row_dft<NX, 1>(a, p.twx, ex, j1);
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(kRowThreads) rows_fwd_kernel(const __grid_cons
 
 template <int NY>
 __global__ void __launch_bounds__(kLatTW<NY> * Lat<NY>::N1) cols_fwd_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
   constexpr int N1 = Lat<NY>::N1, N2 = Lat<NY>::N2, TW = kLatTW<NY>;
   extern __shared__ __align__(16) unsigned char smem[];
   const int pix = threadIdx.x % TW, j1 = threadIdx.x / TW;
@@ -201,6 +203,7 @@ __device__ __forceinline__ float two_sum(float a, float b, float& err) {
 // remainder), which holds 48 bits, and the pairs meet in FP64.  P is scaled by a
 // power of two so that no square leaves the float range.
 __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constant__ ShParams p, size_t n) {
+  after_previous_kernel();
   // two independent sums per thread: one alone waits for its own additions
   float h1[2] = {0.f, 0.f}, l1[2] = {0.f, 0.f}, h2[2] = {0.f, 0.f}, l2[2] = {0.f, 0.f};
   auto add = [&](int k, float v) {
@@ -217,7 +220,7 @@ __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constan
   const size_t n4 = n / 4;
 #pragma unroll 4
   for (size_t i = first; i < n4; i += stride) {
-    const float4 v = __ldg(v4 + i);
+    const float4 v = __ldcs(v4 + i);
     add(0, v.x);
     add(1, v.y);
     add(0, v.z);
@@ -269,6 +272,7 @@ __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constan
 
 template <int NL>
 __global__ void __launch_bounds__(kTile * Split<NL>::N1) axial_adj_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
   constexpr int N1 = Split<NL>::N1, N2 = Split<NL>::N2;
   static_assert(N2 % N1 == 0, "sweep lengths split with N1 | N2");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -309,6 +313,7 @@ __global__ void __launch_bounds__(kTile * Split<NL>::N1) axial_adj_kernel(const 
 
 template <int NY>
 __global__ void __launch_bounds__(kLatTW<NY> * Lat<NY>::N1) cols_adj_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
   constexpr int N1 = Lat<NY>::N1, N2 = Lat<NY>::N2, TW = kLatTW<NY>;
   extern __shared__ __align__(16) unsigned char smem[];
   const int pix = threadIdx.x % TW, j1 = threadIdx.x / TW;
@@ -338,6 +343,7 @@ __global__ void __launch_bounds__(kLatTW<NY> * Lat<NY>::N1) cols_adj_kernel(cons
 
 template <int NX>
 __global__ void __launch_bounds__(kRowThreads) rows_adj_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
   constexpr int N1 = Lat<NX>::N1, N2 = Lat<NX>::N2, RPI = kRowThreads / N1, AS = Lat<NX>::AS;
   extern __shared__ __align__(16) unsigned char smem[];
   const int r = threadIdx.x / N1, j1 = threadIdx.x % N1;
@@ -456,6 +462,7 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 // with two, 33 with four: each thread still ends with some 35 FP64 operations).
 // The reads of Q alone would take 6.
 __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks) {
+  after_previous_kernel();
   const int tx = grid_tx(p.nx), ry = kGradThreads / tx;
   const int x = blockIdx.x * tx + threadIdx.x % tx;
   const size_t npix = (size_t)p.nx * p.ny;
@@ -466,7 +473,7 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
     float qx = 0.f, lx = 0.f, qy = 0.f, ly = 0.f;
 #pragma unroll 16
     for (int c = 0; c < chunks; ++c) {
-      const float2 q = __ldg(p.qpart + (size_t)c * npix + i);
+      const float2 q = __ldcs(p.qpart + (size_t)c * npix + i);
       float e;
       qx = two_sum(qx, q.x, e);
       lx += e;
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
       ly += e;
     }
     // M = -Im(c P Q), the products and their sum as pairs of floats too
-    const float2 cp = __ldg(p.cp + i);
+    const float2 cp = p.cp[i];
     const float u = __fmul_rn(cp.x, qy), v = __fmul_rn(cp.y, qx);
     float e;
     const float h = two_sum(u, v, e);
@@ -536,8 +543,7 @@ cudaError_t launch_k(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  kernel<<<grid, threads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_next(kernel, grid, threads, smem, s, p);
 }
 
 template <int NX>
@@ -652,6 +658,7 @@ constexpr int kPupilRows = 8;  // rows of a block: their polynomials in x come f
 // fmod per pixel that took 78 us at 512 x 512 (two FP64 operations per clock and
 // SM: about 15 per pixel now, 9 us).
 __global__ void __launch_bounds__(256) pupil_table_kernel(const __grid_constant__ PupilParams p) {
+  after_previous_kernel();
   __shared__ double row[kPupilRows][5];
   __shared__ float4 cis[256];
   const int y0 = blockIdx.y * kPupilRows;
@@ -711,8 +718,7 @@ cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s) {
   p.c[3] -= pl.sh_alpha;  // the input chirp, -alpha (dx^2 + dy^2)
   p.c[5] -= pl.sh_alpha;
   const int tx = grid_tx(pl.nx);
-  pupil_table_kernel<<<dim3(pl.nx / tx, (pl.ny + kPupilRows - 1) / kPupilRows), 256, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_next(pupil_table_kernel, dim3(pl.nx / tx, (pl.ny + kPupilRows - 1) / kPupilRows), 256, 0, s, p);
 }
 
 bool generic_lateral_supported(int nx, int ny) {
@@ -778,7 +784,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
   if (e == cudaSuccess && !have_inter) e = cols_any(false, p, s);
   if (e == cudaSuccess) {
-    AxialParams ap;
+    AxialParams ap = {};
     ap.inter = p.inter;
     ap.vol = vol;
     ap.cplx = nullptr;
@@ -793,8 +799,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   }
   const size_t nvox = (size_t)pl.nl * pl.wy * pl.wx;
   if (e == cudaSuccess) {
-    sums_kernel<<<6 * pl.num_sms, kGradThreads, 0, s>>>(p, nvox);
-    e = cudaGetLastError();
+    e = launch_next(sums_kernel, dim3(6 * pl.num_sms), kGradThreads, 0, s, p, nvox);
   }
   if (e == cudaSuccess) e = axial_adj_any(p, s);
   if (e == cudaSuccess) e = cols_any(true, p, s);
@@ -802,8 +807,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   if (e == cudaSuccess) {
     const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;
     const int gy = std::min((p.ny + ry - 1) / ry, std::max(1, 3 * pl.num_sms / gx));
-    grad_kernel<<<dim3(gx, gy), kGradThreads, 0, s>>>(p, chunks);
-    e = cudaGetLastError();
+    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks);
   }
   return e;
 }

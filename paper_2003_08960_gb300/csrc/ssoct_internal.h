@@ -245,6 +245,7 @@ struct AxialParams {
   int nl, wx, wy, ntx;
   float power_scale;       // |K|^2
   int magnitude;           // 1: write |V| instead of |V|^2
+  int late;                // launched after the kernel before it, not beside it (see gate_late)
   unsigned* err;           // error word (kErrAxial), the plan's Counters::err
 };
 
@@ -349,6 +350,8 @@ struct Plan {
 cudaError_t launch_lateral(const Plan& p, const LateralParams& lp, cudaStream_t s);
 cudaError_t launch_axial(const Plan& p, const AxialParams& ap, cudaStream_t s);
 cudaError_t launch_cuts(const CutsParams& cp, cudaStream_t s);
+// Device copy of a multiple of 16 bytes between 16-byte aligned addresses.
+cudaError_t launch_copy_frames(void* dst, const void* src, size_t bytes, cudaStream_t s);
 // The three cuts of the current gate straight from the sweep-axis intermediate
 // (xy: one bin per pixel; xz, yz: the axial transform of the cut's tiles).
 // xy_state, if not NULL, receives the xy cut's complex X(z0) ([wy][ntx * 32]).
@@ -379,6 +382,14 @@ bool lateral_supported(int nx, int ny);
 // launch goes that way.
 int lateral_small_rows(const Plan& p);
 bool lateral_small(const Plan& p);
+// Sliding gates: the kernels that read the intermediate are ordinary launches
+// where it does not fit in L2.  Placed beside the kernel before them (launch_next)
+// the axial kernel took 28 us more at 1024 x 1024 x 256 and the kernels of a
+// cuts-only gate 11 to 23 us more in all (plans in turn, 13 new frames); a gate of
+// 256 x 256 x 128 takes 4 us less so.
+inline bool gate_late(const Plan& p) {
+  return sizeof(float2) * (size_t)p.wy * p.ntx * p.nl * kTile > (128u << 20);
+}
 bool axial_supported(int nl);
 // Tensor-core axial kernel (axial_tc.cu): sweep lengths it handles, its DFT
 // operand table, dynamic shared memory, and launcher.  err is the plan's error

@@ -545,8 +545,12 @@ ssoct_status ssoct_push_frames(ssoct_plan h, const uint16_t* frames, int n, int 
   int done = skip;
   while (done < n) {
     const int run = std::min(n - done, p.nl - p.ring_head);
-    cudaError_t e = cudaMemcpyAsync(p.ws + p.off_ring + fbytes * p.ring_head,
-                                    (const char*)frames + fbytes * done, fbytes * run, kind, s);
+    char* dst = p.ws + p.off_ring + fbytes * p.ring_head;
+    const char* src = (const char*)frames + fbytes * done;
+    // a frame is a multiple of 16 bytes (nx is one of 64 pixels)
+    cudaError_t e = frames_on_device && (uintptr_t)src % 16 == 0
+                        ? launch_copy_frames(dst, src, fbytes * run, s)
+                        : cudaMemcpyAsync(dst, src, fbytes * run, kind, s);
     if (e != cudaSuccess) return cuda_fail(&p, e, "frame copy");
     done += run;
     p.ring_head = (p.ring_head + run) % p.nl;
@@ -638,9 +642,10 @@ static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaSt
   return SSOCT_OK;
 }
 
-static ssoct_status launch_axial_pass(Plan& p, float* vol, void* cplx, cudaStream_t s, cudaEvent_t* ev) {
+static ssoct_status launch_axial_pass(Plan& p, float* vol, void* cplx, bool late, cudaStream_t s, cudaEvent_t* ev) {
   char* ws = p.ws;
   AxialParams ap;
+  ap.late = late ? 1 : 0;
   ap.inter = (const float2*)(ws + p.off_inter);
   ap.vol = vol;
   ap.cplx = (float2*)cplx;
@@ -679,7 +684,7 @@ static ssoct_status run_volume(Plan& p, const uint16_t* frames, int ring_start, 
   cudaEvent_t* ev = nullptr;
   ssoct_status st = launch_lateral_pass(p, lp, s, &ev);
   if (st != SSOCT_OK || p.axial_first) return st;
-  return launch_axial_pass(p, vol, cplx, s, ev);
+  return launch_axial_pass(p, vol, cplx, false, s, ev);
 }
 
 ssoct_status ssoct_reconstruct_volume(ssoct_plan h, float* vol_dev, void* complex_dev, void* stream) {
@@ -753,7 +758,7 @@ ssoct_status ssoct_reconstruct_sliding(ssoct_plan h, float* vol_dev, void* compl
   cudaEvent_t* ev = nullptr;
   ssoct_status st = sliding_update(p, s, &ev);
   if (st != SSOCT_OK) return st;
-  return launch_axial_pass(p, vol_dev, complex_dev, s, ev);
+  return launch_axial_pass(p, vol_dev, complex_dev, gate_late(p), s, ev);
 }
 
 ssoct_status ssoct_sliding_cuts(ssoct_plan h, int x0, int y0, int z0, float* xy, float* xz, float* yz, void* stream) {
