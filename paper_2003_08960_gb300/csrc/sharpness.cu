@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "fft_common.cuh"
+#include "mbarrier.cuh"
 
 namespace ssoct {
 namespace {
@@ -34,7 +35,9 @@ constexpr int kGradThreads = 256;
 // the N1 threads of a transform, stage 2 the N2 N1-point DFTs spread over those
 // threads, NI per thread (the last ones idle when N1 does not divide N2, e.g.
 // 640 = 32 x 20).  AS is the register array length, TW the width of a column
-// tile (16 when 32 N1 threads would exceed 512).
+// tile (16 when 32 N1 threads would exceed 256: at 85 to 128 registers a thread,
+// two or more blocks per SM overlap their loads; loss and gradient at 640 x 384 x
+// 64 446 -> 420 us against tiles of 32, 384 x 384 x 96 380 -> 365).
 template <int N>
 struct Lat {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
@@ -44,7 +47,7 @@ struct Lat {
 // Column-tile width for axis length N (a variable template, instantiated only
 // for the column kernels that use it).
 template <int N>
-constexpr int kLatTW = kTile * Split<N>::N1 <= 512 ? kTile : kTile / 2;
+constexpr int kLatTW = kTile * Split<N>::N1 <= 256 ? kTile : kTile / 2;
 
 __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
 
@@ -389,6 +392,159 @@ __global__ void __launch_bounds__(kRowThreads) rows_adj_kernel(const __grid_cons
 
 }  // namespace
 
+namespace {
+
+// The same row pass, streamed: one CTA per SM takes an equal, contiguous share of
+// the (band of rows, frame) pairs, band by band, and its inputs (the band's rows of
+// F, the raw frame rows and the taps of Eq. 5) arrive by bulk copies into two stage
+// buffers, one pair ahead.  rows_adj_kernel's accumulators leave room for eight
+// warps per SM, which wait for each of these loads in turn.  The exchange is done
+// in place in the stage buffer.  A CTA writes its share of a band's sum to partial
+// sum (its rank among the band's CTAs).  Loss and gradient at 512 x 512 x 128 726 ->
+// 683 us, 1024 x 1024 x 64 1404 -> 1279, 768 x 768 x 64 887 -> 825, 256 x 256 x 256
+// 488 -> 427.  Column and row passes in turn over chunks of frames whose F stays in
+// L2 were slower (16 to 96 MiB: 724 to 767 us at 512 x 512 x 128).
+struct RowsAdjShare {
+  int bands, nt, ctas;
+  __host__ __device__ long long pairs() const { return (long long)bands * nt; }
+  __host__ __device__ int first(int c) const { return (int)(pairs() * c / ctas); }  // first pair of CTA c
+  // CTA of pair i, and the number of partial sums of a band
+  __host__ __device__ int cta_of(int i) const { return (int)((((long long)i + 1) * ctas - 1) / pairs()); }
+  __host__ __device__ int slots(int band) const { return cta_of((band + 1) * nt - 1) - cta_of(band * nt) + 1; }
+};
+
+template <int NX>
+struct RowsAdjStage {
+  static constexpr int RPI = kRowThreads / Lat<NX>::N1;
+  static constexpr size_t kRows = (size_t)RPI * NX * sizeof(float2);  // then the raw rows, x taps, y taps
+  __host__ __device__ static size_t taps_at(int raw_rows) { return kRows + (size_t)raw_rows * NX * sizeof(uint16_t); }
+  __host__ __device__ static size_t bytes(int raw_rows) { return taps_at(raw_rows) + NX * sizeof(Tap) + RPI * sizeof(Tap); }
+};
+
+constexpr unsigned long long kAdjWaitNs = 4000000000ull;  // 4 s
+
+template <int NX>
+__global__ void __launch_bounds__(kRowThreads, 1)
+    rows_adj_stream_kernel(const __grid_constant__ ShParams p, RowsAdjShare share, int raw_rows, unsigned* err) {
+  after_previous_kernel();
+  using St = RowsAdjStage<NX>;
+  constexpr int N1 = Lat<NX>::N1, N2 = Lat<NX>::N2, NI = Lat<NX>::NI, RPI = St::RPI, AS = Lat<NX>::AS;
+  static_assert(32 % N1 == 0, "a row's N1 threads lie in one warp");
+  extern __shared__ __align__(1024) unsigned char smem_adj[];
+  __shared__ __align__(8) uint64_t full[2];
+  const int tid = threadIdx.x;
+  const int r = tid / N1, j1 = tid % N1;
+  const size_t stage_bytes = (St::bytes(raw_rows) + 127) / 128 * 128;
+  const size_t taps_at = St::taps_at(raw_rows);
+  const int lo = share.first(blockIdx.x), hi = share.first(blockIdx.x + 1);
+  // pair i into stage buffer (i - lo) mod 2, by one thread
+  auto fill = [&](int i) {
+    const int band = i / share.nt, t = i - band * share.nt;
+    unsigned char* buf = smem_adj + (size_t)((i - lo) & 1) * stage_bytes;
+    uint64_t* bar = &full[(i - lo) & 1];
+    const Tap* yt = p.ytab + (size_t)t * p.ny + band * RPI;
+    const int first = yt[0].base, rows = yt[RPI - 1].base + 2 - first;  // at most raw_rows
+    const unsigned raw = (unsigned)(rows * NX * sizeof(uint16_t));
+    mbar_arrive_tx(bar, (unsigned)St::kRows + raw + (unsigned)((NX + RPI) * sizeof(Tap)));
+    tma_load_1d(buf, p.F + ((size_t)t * p.ny + band * RPI) * NX, (unsigned)St::kRows, bar);
+    tma_load_1d(buf + St::kRows, p.frames + ((size_t)((p.ring_start + t) % p.nl) * p.ny + first) * NX, raw, bar);
+    tma_load_1d(buf + taps_at, p.xtab + (size_t)t * NX, (unsigned)(NX * sizeof(Tap)), bar);
+    tma_load_1d(buf + taps_at + NX * sizeof(Tap), yt, (unsigned)(RPI * sizeof(Tap)), bar);
+  };
+  // bounded wait for the CTA's k-th pair
+  auto arrived = [&](int k) {
+    uint64_t* bar = &full[k & 1];
+    const unsigned parity = (unsigned)(k / 2) & 1u;
+    if (mbar_try(bar, parity)) return true;
+    const unsigned long long since = global_timer_ns();
+    while (!mbar_try(bar, parity))
+      if (global_timer_ns() - since > kAdjWaitNs) return false;
+    return true;
+  };
+  if (tid == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = lo; i < hi && i < lo + 2; ++i) fill(i);
+  }
+  __syncthreads();
+  float2 acc[AS];
+#pragma unroll
+  for (int i = 0; i < AS; ++i) acc[i] = make_float2(0.f, 0.f);
+  for (int i = lo; i < hi; ++i) {
+    const int k = i - lo;
+    const bool ok = arrived(k);
+    if (__syncthreads_or(!ok)) {
+      // the copies never came: the sums are incomplete, and reported so; what is
+      // still in flight lands before the CTA exits
+      if (tid == 0) {
+        atomicOr(err, kErrAxial);
+        arrived(k);
+        if (i + 1 < hi) arrived(k + 1);
+      }
+      return;
+    }
+    unsigned char* buf = smem_adj + (size_t)(k & 1) * stage_bytes;
+    float2* row = reinterpret_cast<float2*>(buf) + r * NX;
+    const uint16_t* raw = reinterpret_cast<const uint16_t*>(buf + St::kRows);
+    const Tap* xt = reinterpret_cast<const Tap*>(buf + taps_at);
+    float2 a[AS];
+#pragma unroll
+    for (int j2 = 0; j2 < N2; ++j2) a[j2] = row[j1 + N1 * j2];
+    Dft<N2, -1>::template run<1, 0>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) a[k2] = cmul(a[k2], conjf2(ldg2(p.twx + k2 * N1 + j1)));
+    __syncwarp();  // the row's values have been read
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) row[k2 * N1 + (j1 ^ (k2 & (N1 - 1)))] = a[k2];
+    __syncwarp();
+    const Tap ty = xt[NX + r];
+    const uint16_t* r0 = raw + (ty.base - xt[NX].base) * NX;
+    static_for<0, NI>([&](auto I) {
+      constexpr int ii = decltype(I)::value;
+      const int k2 = j1 + N1 * ii;
+      if (N2 % N1 == 0 || k2 < N2) {
+#pragma unroll
+        for (int jj = 0; jj < N1; ++jj) a[ii * N1 + jj] = row[k2 * N1 + (jj ^ (k2 & (N1 - 1)))];
+        Dft<N1, -1>::template run<1, ii * N1>(a);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+          const Tap tx = xt[k2 + N2 * k1];
+          const uint16_t* c = r0 + tx.base;
+          const float v0 = fmaf(tx.w0, (float)c[0], tx.w1 * (float)c[1]);
+          const float v1 = fmaf(tx.w0, (float)c[NX], tx.w1 * (float)c[NX + 1]);
+          const float u = fmaf(ty.w0, v0, ty.w1 * v1);
+          const float2 v = a[ii * N1 + k1];
+          acc[ii * N1 + k1].x = fmaf(v.x, u, acc[ii * N1 + k1].x);   // conj(Y) u
+          acc[ii * N1 + k1].y = fmaf(-v.y, u, acc[ii * N1 + k1].y);
+        }
+      }
+    });
+    // this thread's accesses to the buffer come before its next fill (async proxy)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0 && i + 2 < hi) fill(i + 2);
+    const int band = i / share.nt;
+    if (i + 1 == hi || (i + 1) / share.nt != band) {
+      const int slot = (int)blockIdx.x - share.cta_of(band * share.nt);
+      float2* dst = p.qpart + ((size_t)slot * p.ny + band * RPI + r) * NX;
+      static_for<0, NI>([&](auto I) {
+        constexpr int ii = decltype(I)::value;
+        const int k2 = j1 + N1 * ii;
+        if (N2 % N1 == 0 || k2 < N2) {
+#pragma unroll
+          for (int k1 = 0; k1 < N1; ++k1) {
+            dst[k2 + N2 * k1] = acc[ii * N1 + k1];
+            acc[ii * N1 + k1] = make_float2(0.f, 0.f);
+          }
+        }
+      });
+    }
+  }
+}
+
+}  // namespace
+
 // Z_1..Z_15 (Noll order, RMS-normalised on the unit disk; Noll 1976) at radius
 // rho and angle (cos th, sin th).
 __host__ __device__ __forceinline__ void zernike15(double rho, double c1, double s1, double (&z)[15]) {
@@ -461,7 +617,8 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 // clock and SM) took 98 us at 512 x 512 x 128; 31 us now (three blocks per SM; 36
 // with two, 33 with four: each thread still ends with some 35 FP64 operations).
 // The reads of Q alone would take 6.
-__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks) {
+__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks,
+                                                           RowsAdjShare share, int band_rows) {
   after_previous_kernel();
   const int tx = grid_tx(p.nx), ry = kGradThreads / tx;
   const int x = blockIdx.x * tx + threadIdx.x % tx;
@@ -471,8 +628,9 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
   for (int y = blockIdx.y * ry + threadIdx.x / tx; y < p.ny; y += gridDim.y * ry) {
     const size_t i = (size_t)y * p.nx + x;
     float qx = 0.f, lx = 0.f, qy = 0.f, ly = 0.f;
-#pragma unroll 16
-    for (int c = 0; c < chunks; ++c) {
+    const int parts = band_rows ? share.slots(y / band_rows) : chunks;
+#pragma unroll 8
+    for (int c = 0; c < parts; ++c) {
       const float2 q = __ldcs(p.qpart + (size_t)c * npix + i);
       float e;
       qx = two_sum(qx, q.x, e);
@@ -598,6 +756,27 @@ cudaError_t cols_any(bool adj, const ShParams& p, cudaStream_t s) {
     case 768: return cols<768>(adj, p, s);
     case 1024: return cols<1024>(adj, p, s);
   }
+  return cudaErrorInvalidValue;
+}
+
+size_t rows_adj_stream_smem(const Plan& pl) {
+#define X(n) if (pl.nx == n) return 2 * ((RowsAdjStage<n>::bytes(pl.stage_rows) + 127) / 128 * 128);
+  X(64) X(128) X(256) X(384) X(512) X(640) X(768) X(1024)
+#undef X
+  return SIZE_MAX;
+}
+
+cudaError_t rows_adj_stream_any(const ShParams& p, const RowsAdjShare& share, int raw_rows, unsigned* err, cudaStream_t s) {
+#define X(n)                                                                                                        \
+  if (p.nx == n) {                                                                                                  \
+    const size_t smem = 2 * ((RowsAdjStage<n>::bytes(raw_rows) + 127) / 128 * 128);                                 \
+    const cudaError_t e = cudaFuncSetAttribute(rows_adj_stream_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                               (int)smem);                                                          \
+    if (e != cudaSuccess) return e;                                                                                 \
+    return launch_next(rows_adj_stream_kernel<n>, dim3(share.ctas), kRowThreads, smem, s, p, share, raw_rows, err); \
+  }
+  X(64) X(128) X(256) X(384) X(512) X(640) X(768) X(1024)
+#undef X
   return cudaErrorInvalidValue;
 }
 
@@ -802,12 +981,21 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     e = launch_next(sums_kernel, dim3(6 * pl.num_sms), kGradThreads, 0, s, p, nvox);
   }
   if (e == cudaSuccess) e = axial_adj_any(p, s);
+  // The adjoint row pass is streamed where every SM gets two pairs or more, the
+  // partial sums suffice (a band has at most ctas / bands + 2) and bulk copies can
+  // read the frames.
+  const int band_rows = kRowThreads / pl.n1x;
+  const RowsAdjShare share{pl.ny / band_rows, pl.nl, pl.num_sms};
+  const bool stream = (uintptr_t)frames % 16 == 0 && share.pairs() >= 2ll * share.ctas &&
+                      share.ctas <= (long long)share.bands * (chunks - 2) && rows_adj_stream_smem(pl) <= 226u * 1024u;
   if (e == cudaSuccess) e = cols_any(true, p, s);
-  if (e == cudaSuccess) e = rows_any(true, p, chunks, s);
+  if (e == cudaSuccess)
+    e = stream ? rows_adj_stream_any(p, share, pl.stage_rows, &((Counters*)(ws + pl.off_ctr))->err, s)
+               : rows_any(true, p, chunks, s);
   if (e == cudaSuccess) {
     const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;
     const int gy = std::min((p.ny + ry - 1) / ry, std::max(1, 3 * pl.num_sms / gx));
-    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks);
+    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks, share, stream ? band_rows : 0);
   }
   return e;
 }

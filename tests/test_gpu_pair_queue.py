@@ -62,3 +62,25 @@ def test_aberration_path_from_any_alignment(window):
     assert float((v0.double() - v1.double()).norm()) <= 2e-5 * float(v1.double().norm())
     assert abs(l0 - l1) <= 2e-5 * abs(l1)
     assert np.linalg.norm(g0[1:] - g1[1:]) <= 2e-4 * np.linalg.norm(g1[1:])
+
+
+# streamed adjoint row pass (aligned frames) against the plain one (any alignment):
+# bands that end inside a CTA's share, mixed-radix rows, a band of eight rows, the
+# last share shorter
+@pytest.mark.parametrize("shape,window", [((256, 256, 128), (30, 7, 101, 200)), ((640, 384, 64), None),
+                                          ((1024, 64, 200), (1, 3, 1000, 55)), ((384, 256, 160), None)])
+def test_adjoint_rows_streamed_and_plain(shape, window):
+    import paper_2003_08960_gb300 as ss
+    nx, ny, nl = shape
+    lam = synth.interferograms.sweep_wavelengths(800e-9, 850e-9, nl)
+    plan = ss.Plan(nx, ny, nl, 20e-6, 0.3, lam, window=window, flags=ss.SSOCT_FLAG_PUPIL)
+    aligned = torch.from_numpy(_frames(shape, nx * nl).view(np.int16)).cuda()
+    flat = torch.empty(aligned.numel() + 1, dtype=torch.int16, device="cuda")
+    flat[1:] = aligned.reshape(-1)
+    coeffs = (0.2 * np.random.default_rng(nl).standard_normal(15)).tolist()
+    l0, g0, _ = plan.sharpness(aligned, coeffs, 0.301)
+    l1, g1, _ = plan.sharpness(flat[1:].view(aligned.shape), coeffs, 0.301)
+    # two FP32 evaluations of the same sums
+    assert abs(l0 - l1) <= 2e-5 * abs(l1)
+    assert np.linalg.norm(g0[1:] - g1[1:]) <= 2e-4 * np.linalg.norm(g1[1:])
+    assert abs(g0[0] - g1[0]) <= 2e-4 * np.linalg.norm(g1)
