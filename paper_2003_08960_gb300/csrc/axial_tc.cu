@@ -30,7 +30,16 @@
 // stage-2 operands overwrite those once the stage-1 MMAs are done, and the
 // |V|^2 rows overwrite those once the stage-2 MMAs are done.  Each group owns
 // 64 TMEM columns (2 blocks x N = 32 fp32 accumulators); one of its threads
-// issues its 12 MMAs per stage and waits on its commit barrier.
+// issues its 12 MMAs per stage, and every thread waits on its commit barrier.
+//
+// The rows leave by one tensor copy per half-tile (256 depth bins x 16 pixels,
+// clipped at the window), which the group does not wait for: the buffer is refilled
+// in the middle of the group's next half-tile.  What bounds the kernel is that the
+// groups wait for one another's steps, so the steps were made fewer: four group
+// barriers a half-tile instead of eight, and no copy of the rows through registers.
+// 512x512x256: 175 -> 159 us (805 MB, 5.1 TB/s), 1024x1024x256: 656 -> 594 us
+// (3.2 GB, 5.4 TB/s).  Stores straight from tensor memory in 32-byte pieces had
+// been slower (720 us against 657 at the time).
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -112,7 +121,7 @@ __device__ __forceinline__ void tc_ld32(unsigned taddr, float (&v)[32]) {
 }
 // Bounded wait for an mbarrier phase (true on completion).
 __device__ bool tc_wait(uint64_t* bar, unsigned parity, unsigned long long limit_ns = kTcWaitNs) {
-  const unsigned long long t0 = global_timer_ns();
+  unsigned long long t0 = 0;
   for (;;) {
     unsigned ok;
     asm volatile(
@@ -121,7 +130,9 @@ __device__ bool tc_wait(uint64_t* bar, unsigned parity, unsigned long long limit
         : "r"(smem_addr(bar)), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (global_timer_ns() - t0 > limit_ns) return false;
+    const unsigned long long now = global_timer_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) return false;
   }
 }
 
@@ -138,6 +149,7 @@ struct TcParams {
   float k_abs;                  // |K|, folded into the stage-2 twiddles (so |V|^2 |K|^2 = |v|^2)
   float inv_k_abs;              // 1 / |K|, taken back out of the complex output (oy holds K)
   int magnitude;
+  int bulk;                     // rows leave by tensor copies (vmap)
   unsigned* err;                // kErrAxialTc (MMA wait) / kErrAxial (tile wait) ORed in on a time-out
 };
 
@@ -152,6 +164,12 @@ __device__ __forceinline__ void split2_bf16(float a, float b, unsigned& hi, unsi
 // Row of the M = 128 operand block for (8-pixel block entry pl, radix index i):
 // i * 8 + pl keeps a warp's 32 pixels on distinct 16-byte slots of a core matrix.
 __device__ __forceinline__ int tc_row(int i, int pl) { return i * 8 + pl; }
+// Stage 2 puts k2 in place i with bits 1 and 2 exchanged (its own inverse): a
+// warp's four k2 then differ in bits 0 and 2, and its 32 |V|^2 values lie in 32
+// banks of the swizzled output rows.
+__host__ __device__ __forceinline__ constexpr int tc_k2_row(int k2) {
+  return (k2 & 9) | ((k2 & 2) << 1) | ((k2 & 4) >> 1);
+}
 
 // Barrier of one group (named barrier 1 + g, 256 threads); returns the OR of v.
 __device__ __forceinline__ bool tc_group_sync_or(int g, bool v) {
@@ -174,7 +192,6 @@ __device__ __forceinline__ void tc_tma_2d(void* dst, const CUtensorMap* map, int
 }
 
 constexpr int kABlock = 128 * kTcK;  // elements of one M block of an operand
-constexpr int kOutStride = 24;       // floats per |V|^2 row in the buffer: conflict-free writes
 
 // Copy of the CTA's work item t (global item blockIdx.x + t * gridDim.x: half
 // item % 2 of tile item / 2) into ring buffer t mod kTcStages.  The tensor map
@@ -210,6 +227,12 @@ __device__ __forceinline__ void tc_issue_stage(unsigned tmem, const unsigned sho
   tc_commit(bar);
 }
 
+// Place of depth bin q, pixel px in the item's |V|^2 rows (16 floats a row), in
+// the 64-byte swizzle of tensor copies: 16-byte chunk number XOR (row / 2) mod 4.
+__device__ __forceinline__ int tc_out(int q, int px) {
+  return q * kTcHalf + ((((px >> 2) ^ (q >> 1)) & 3) << 2) + (px & 3);
+}
+
 // |V|^2 |K|^2 (|V| |K| if MAG) of the 16 depth bins q = k2 + 16 k1 this thread
 // holds (v carries |K| from the twiddles) into the item's output rows; with
 // CPLX also V with the output chirp and K.
@@ -222,21 +245,22 @@ __device__ __forceinline__ void tc_epilogue(const TcParams& p, const float (&v)[
     if (in) of = cmul(ldg2(p.ox + kx0 + px), ldg2(p.oy + kyw));
     of = make_float2(of.x * p.inv_k_abs, of.y * p.inv_k_abs);
   }
+  out += tc_out(k2, px);  // 16 rows on, the swizzle is the same
 #pragma unroll
   for (int k1 = 0; k1 < 16; ++k1) {
-    const int q = k2 + 16 * k1;
     const float2 x = make_float2(v[2 * k1], v[2 * k1 + 1]);
     float pw = fmaf(x.x, x.x, x.y * x.y);
     if constexpr (MAG) pw = sqrtf(pw);
-    out[q * kOutStride + px] = pw;
+    out[k1 * 16 * kTcHalf] = pw;
     if constexpr (CPLX) {
-      if (in) __stcs(p.cplx + ((size_t)q * p.wy + kyw) * p.wx + kx0 + px, cmul(x, of));
+      if (in) __stcs(p.cplx + ((size_t)(k2 + 16 * k1) * p.wy + kyw) * p.wx + kx0 + px, cmul(x, of));
     }
   }
 }
 
 __global__ void __launch_bounds__(kTcThreads, 1)
-    axial_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap imap) {
+    axial_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap imap,
+                    const __grid_constant__ CUtensorMap vmap) {
   after_previous_kernel();
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* ring = smem;                                                      // [6][32 KB]
@@ -278,17 +302,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int gw = lt / 32;                       // warp within the group (0..7)
   const int quad = gw & 3, qblk = gw >> 2;      // TMEM lane quadrant, M block read by this warp
   const unsigned tmem = tmem_base + (unsigned)(g * kTcCols);
-  for (int i = g, prev = -1;; prev = i, i += kTcGroups) {
-    tc_group_sync(g);  // every thread of the group is done with item prev's buffer
-    if (lt == 0 && prev >= 0 && prev + kTcStages < mine) tc_fill(&imap, ring, full, fills, prev + kTcStages);
-    if (i >= mine) break;
-    // one thread waits for the item; the others sleep at the group barrier
-    bool ok0 = true;
-    if (lt == 0) {
-      ok0 = tc_wait(&full[i % kTcFull], (unsigned)(i / kTcFull) & 1u, kTcLoadWaitNs);
-      if (!ok0) atomicOr(p.err, kErrAxial);
+  // A wait that runs out is agreed on at the group's next barrier, so that no
+  // thread of a group leaves the loop alone.
+  bool bad = false;
+  for (int i = g, prev = -1; i < mine; prev = i, i += kTcGroups) {
+    if (!tc_wait(&full[i % kTcFull], (unsigned)(i / kTcFull) & 1u, kTcLoadWaitNs)) {
+      atomicOr(p.err, kErrAxial);
+      bad = true;
     }
-    if (tc_group_sync_or(g, !ok0)) break;
     unsigned char* buf = ring + (size_t)(i % kTcStages) * kTcItemBytes;
     unsigned short* A = reinterpret_cast<unsigned short*>(buf);  // [hi / lo][block][128 x 32]
     const int gi = (int)blockIdx.x + i * (int)gridDim.x;
@@ -310,7 +331,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int k = 0; k < 8; ++k) x[u][k] = src[(j1 + 16 * (8 * h + k)) * kTcHalf];
       }
-      tc_group_sync(g);
+      if (tc_group_sync_or(g, bad)) break;
+      // item prev's rows have left its buffer, or nearly: refill it
+      if (lt == 0 && prev >= 0 && prev + kTcStages < mine) {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        tc_fill(&imap, ring, full, fills, prev + kTcStages);
+      }
       const int blk = px >> 3, pl = px & 7;
       unsigned short* Ahi = A + blk * kABlock;
       unsigned short* Alo = A + (kTcItemBlocks + blk) * kABlock;
@@ -338,16 +364,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_before();
     tc_group_sync(g);
     tc_fence_after();
-    bool ok = true;
-    if (lt == 0) {
-      tc_issue_stage(tmem, A, Bs, &mma_bar[g]);
-      ok = tc_wait(&mma_bar[g], 0u);
-      if (!ok) atomicOr(p.err, kErrAxialTc);
+    if (lt == 0) tc_issue_stage(tmem, A, Bs, &mma_bar[g]);
+    __syncwarp();
+    if (!tc_wait(&mma_bar[g], 0u)) {
+      atomicOr(p.err, kErrAxialTc);
+      bad = true;
     }
-    tc_fence_before();
-    const bool bad1 = tc_group_sync_or(g, !ok);
+    __syncwarp();  // tcgen05.ld is issued by whole warps
     tc_fence_after();
-    if (bad1) break;
 
     // 2. twiddle w256^(j1 k2) and re-layout as the stage-2 operand: row (pixel, k2),
     //    K = 2 j1 (real) / 2 j1 + 1 (imaginary), over the stage-1 operand (its MMAs are done)
@@ -361,7 +385,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int k2 = 0; k2 < 16; ++k2) {
         const float2 z = cmul(make_float2(v[2 * k2], v[2 * k2 + 1]), tw[k2 * 16 + j1]);
-        const int off = tc_core_off(tc_row(k2, pl), 2 * j1);
+        const int off = tc_core_off(tc_row(tc_k2_row(k2), pl), 2 * j1);
         unsigned hi, lo;
         split2_bf16(z.x, z.y, hi, lo);
         *reinterpret_cast<unsigned*>(Ahi + off) = hi;
@@ -370,26 +394,26 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
-    tc_group_sync(g);
+    const bool bad1 = tc_group_sync_or(g, bad);
     tc_fence_after();
-    if (lt == 0) {
-      tc_issue_stage(tmem, A, Bs, &mma_bar[g]);
-      ok = tc_wait(&mma_bar[g], 1u);
-      if (!ok) atomicOr(p.err, kErrAxialTc);
+    if (bad1) break;
+    if (lt == 0) tc_issue_stage(tmem, A, Bs, &mma_bar[g]);
+    __syncwarp();
+    if (!tc_wait(&mma_bar[g], 1u)) {
+      atomicOr(p.err, kErrAxialTc);
+      bad = true;
     }
-    tc_fence_before();
-    const bool bad2 = tc_group_sync_or(g, !ok);
+    __syncwarp();  // tcgen05.ld is issued by whole warps
     tc_fence_after();
-    if (bad2) break;
 
     // 3. V[k2 + 16 k1] sits in row (pixel, k2), columns 2 k1 (real) / 2 k1 + 1
     //    (imaginary); |V|^2 rows over the stage-2 operand (its MMAs are done)
-    float* out = reinterpret_cast<float*>(buf);  // [256][kOutStride]
+    float* out = reinterpret_cast<float*>(buf);  // [256][16], tc_out
     {
       float v[32];
       tc_ld32(tmem + ((unsigned)(quad * 32) << 16) + (unsigned)(qblk * kTcK), v);
       const int r = quad * 32 + lane;
-      const int k2 = r >> 3, px = qblk * 8 + (r & 7);
+      const int k2 = tc_k2_row(r >> 3), px = qblk * 8 + (r & 7);
       if (p.cplx) {
         if (p.magnitude) tc_epilogue<true, true>(p, v, out, k2, px, kx0, kyw);
         else tc_epilogue<false, true>(p, v, out, k2, px, kx0, kyw);
@@ -398,22 +422,31 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         else tc_epilogue<false, false>(p, v, out, k2, px, kx0, kyw);
       }
     }
-    tc_group_sync(g);
-    // 4. 64-byte rows of the volume: per pass 16 depth bins, a warp's two halves
-    //    on bins two apart (distinct banks with the 24-float row stride)
-    {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (tc_group_sync_or(g, bad)) break;
+    // 4. 64-byte rows of the volume
+    if (p.bulk) {
+      if (lt == 0 && kx0 < p.wx) {  // columns beyond wx are clipped by the copy
+        asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(&vmap),
+                     "r"(kx0), "r"(kyw), "r"(0), "r"(smem_addr(buf))
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      }
+      __syncwarp();
+    } else {
+      // per pass 16 depth bins, a warp's two halves on adjacent ones (distinct banks)
       const int px = lane & (kTcHalf - 1);
-      const int qa = (gw & 1) + 4 * (gw >> 1) + 2 * (lane >> 4);
       if (kx0 + px < p.wx) {
         float* dst = p.vol + (size_t)kyw * p.wx + kx0 + px;
         const size_t plane = (size_t)p.wy * p.wx;
 #pragma unroll 4
-        for (int q = qa; q < kTcN; q += 16) __stcs(dst + (size_t)q * plane, out[q * kOutStride + px]);
+        for (int q = 2 * gw + (lane >> 4); q < kTcN; q += 16) __stcs(dst + (size_t)q * plane, out[tc_out(q, px)]);
       }
+      // these reads come before the buffer's next fill (async proxy)
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // this thread's accesses to the buffer come before its next TMA fill (async proxy)
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (lt == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   // copies still in flight (after a time-out) land before the CTA exits; the
   // last fill of each barrier is its latest phase
   tc_fence_before();
@@ -494,12 +527,18 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
   if (e != cudaSuccess) return e;
   alignas(64) CUtensorMap imap;
   if (!encode_inter_map(ap.inter, (long long)ap.ntx * ap.wy * kTcN, kTcHalf, &imap)) return cudaErrorInvalidValue;
+  // A tensor copy needs rows on 16-byte boundaries (volumes are); every other width
+  // takes 64-byte runs from its threads (512x512x256 with a window of
+  // 333 x 400: 104.8 us, of 332 x 400 by tensor copies: 93.3 us).
+  alignas(64) CUtensorMap vmap = {};
+  p.bulk = ap.wx % 4 == 0;
+  if (p.bulk && !encode_volume_map(ap.vol, ap.wx, ap.wy, kTcN, kTcHalf, &vmap)) return cudaErrorInvalidValue;
   const long long nitems = 2ll * ap.ntx * ap.wy;
   long long grid = num_sms > 0 ? num_sms : 1;  // persistent: one CTA per SM
   if (grid > nitems) grid = nitems;
   if (grid < 1) return cudaSuccess;
-  return ap.late ? launch_after(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap)
-                 : launch_next(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap);
+  return ap.late ? launch_after(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap, vmap)
+                 : launch_next(axial_tc_kernel, dim3((unsigned)grid), kTcThreads, smem, s, p, imap, vmap);
 }
 
 }  // namespace ssoct

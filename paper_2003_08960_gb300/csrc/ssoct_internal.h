@@ -376,6 +376,10 @@ bool encode_frames_map(const Plan& p, const uint16_t* frames, int box_cols, void
 // row = 32 complex values of one frame of a tile), boxes of box_complex
 // complex values x 256 rows.
 bool encode_inter_map(const float2* inter, long long rows, int box_complex, void* map_out);
+// Tensor map over a volume float [nl][wy][wx] (wx a multiple of 4, vol 16-byte
+// aligned), boxes of box_px pixels of one row x nl depth bins (at most 256), whose
+// shared-memory rows of 64 bytes (box_px 16) are in the 64-byte swizzle.
+bool encode_volume_map(float* vol, int wx, int wy, int nl, int box_px, void* map_out);
 bool lateral_supported(int nx, int ny);
 // Frames that one CTA or cluster transforms whole, without the work queue: the
 // raw rows that a CTA's band takes (0: not such a plan), and whether the next

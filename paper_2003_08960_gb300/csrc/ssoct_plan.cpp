@@ -140,6 +140,19 @@ bool encode_inter_map(const float2* inter, long long rows, int box_complex, void
   return r == CUDA_SUCCESS;
 }
 
+bool encode_volume_map(float* vol, int wx, int wy, int nl, int box_px, void* map_out) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)wx, (cuuint64_t)wy, (cuuint64_t)nl};
+  cuuint64_t strides[2] = {(cuuint64_t)wx * sizeof(float), (cuuint64_t)wx * wy * sizeof(float)};
+  cuuint32_t box[3] = {(cuuint32_t)box_px, 1, (cuuint32_t)nl};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(reinterpret_cast<CUtensorMap*>(map_out), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, vol, dims, strides,
+                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 bool encode_frames_map(const Plan& p, const uint16_t* frames, int box_cols, void* map_out) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
