@@ -212,6 +212,40 @@ __device__ __forceinline__ void row_item(const LateralParams& p, const Desc& d, 
   float2* ex = reinterpret_cast<float2*>(buf) + r * NX;  // this row's block (N2 x N1 = NX values)
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) ex[xswz<N1>(k2, j1)] = a[k2];
+  if constexpr (N2 % N1 != 0) {
+    // The group's RPI x N2 second-stage DFTs are dealt out to its threads in order, so
+    // that whole warps are idle and not 8 to 12 lanes of every warp (of 8 warps 5 work
+    // for 640, 6 for 768; 12 of 16 turns for 384), at the price of the group's barrier;
+    // fewer live registers, too (640: 104 -> 32 bytes of spills).  Group 1 begins
+    // two warps on, which puts the two groups' odd warps on different schedulers.
+    // Lateral time, us, before / after: 640 x 640 x 160 351 / 319 (with a 400 x 300
+    // window 367 / 343), 768 x 768 x 200 573 / 541, 384 x 384 x 96 75 / 68, 384 x 640 x
+    // 160 250 / 237, 640 x 384 x 160 251 / 251.
+    consumers_sync(g);
+    constexpr int kDfts = RPI * N2;
+    const unsigned long long pol_last = policy_evict_last();
+    float2* slot = p.scratch + ((size_t)(f % p.sch.slots) * p.ny + d.item * RPI) * p.wxp;
+    static_for<0, (kDfts + kThreads - 1) / kThreads>([&](auto I) {
+      const int t = ((tid - 64 * g) & (kThreads - 1)) + kThreads * decltype(I)::value;
+      const int rr = t / N2, k2 = t - rr * N2;
+      if (t >= kDfts) return;
+      const float2* from = reinterpret_cast<const float2*>(buf) + rr * NX;
+#pragma unroll
+      for (int jj = 0; jj < N1; ++jj) a[jj] = from[xswz<N1>(k2, jj)];
+      Dft<N1, 1>::template run<1, 0>(a);
+      float2* dst = slot + (size_t)rr * p.wxp;
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) {
+        if constexpr (FW) {
+          st_cg_hint(dst + k2 + N2 * k1, a[k1], pol_last);
+        } else {
+          const int kw = k2 + N2 * k1 - p.x0;
+          if (kw >= 0 && kw < p.wx) st_cg_hint(dst + kw, a[k1], pol_last);
+        }
+      }
+    });
+    return;
+  }
   __syncwarp();  // a row's N1 threads lie in one warp
   static_for<0, S2::NI>([&](auto I) {
     constexpr int i = decltype(I)::value;
@@ -316,10 +350,13 @@ __device__ __forceinline__ void col_item(const LateralParams& p, const Desc& d, 
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) tile[col_row<N1, BC>(j1, k2) * BC + b] = a[k2];
   consumers_sync(g);
+  // where some of the group's warps are idle in the whole second stage, other ones in
+  // the two groups, as in row_item (640 x 640 x 160 with a window 348 -> 343 us)
+  const int jc = N2 < N1 ? ((tid - 64 * g) & (kThreads - 1)) / BC : j1;
   static_for<0, S2::NI>([&](auto I) {
     constexpr int i = decltype(I)::value;
-    const int k2 = j1 + N1 * i;
-    if (!S2::live(i, j1)) return;
+    const int k2 = jc + N1 * i;
+    if (!S2::live(i, jc)) return;
     if constexpr (BC == 8) {
       // row jj ^ sw: jj + sw for even jj, jj - sw for odd jj (two bases, constant offsets)
       const int sw = k2 & 1;
@@ -341,11 +378,11 @@ __device__ __forceinline__ void col_item(const LateralParams& p, const Desc& d, 
     const int kxw = d.item * BC + b;  // column bands already span the window's columns
     if (kxw < p.wx) {
       if (p.cplx) {
-        if (p.magnitude) af_epilogue<NY, FW, true, true, NX>(p, d, a, j1, kxw);
-        else af_epilogue<NY, FW, false, true, NX>(p, d, a, j1, kxw);
+        if (p.magnitude) af_epilogue<NY, FW, true, true, NX>(p, d, a, jc, kxw);
+        else af_epilogue<NY, FW, false, true, NX>(p, d, a, jc, kxw);
       } else {
-        if (p.magnitude) af_epilogue<NY, FW, true, false, NX>(p, d, a, j1, kxw);
-        else af_epilogue<NY, FW, false, false, NX>(p, d, a, j1, kxw);
+        if (p.magnitude) af_epilogue<NY, FW, true, false, NX>(p, d, a, jc, kxw);
+        else af_epilogue<NY, FW, false, false, NX>(p, d, a, jc, kxw);
       }
     }
   } else {
@@ -356,8 +393,8 @@ __device__ __forceinline__ void col_item(const LateralParams& p, const Desc& d, 
       const size_t row_pitch = (size_t)p.ntx * p.nl * kTile;
       static_for<0, S2::NI>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        const int k2 = j1 + N1 * i;
-        if (!S2::live(i, j1)) return;
+        const int k2 = jc + N1 * i;
+        if (!S2::live(i, jc)) return;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) {
           if constexpr (FW) {

@@ -44,6 +44,30 @@ def test_non_square_frames(shape, window, last):
     assert np.all(np.abs(vol.cpu().numpy().astype(np.float64) - oracle.intensity(ref)) <= 2 * e * np.abs(ref) + e * e)
 
 
+# rows whose second-stage transforms are dealt out over a group's threads: whole rows,
+# and windows that begin or end inside a thread's run of outputs
+@pytest.mark.parametrize("n", [384, 640, 768])
+@pytest.mark.parametrize("axial_first", [False, True])
+@pytest.mark.parametrize("crop", [None, (0, 0, 1, 3), (19, 23, 33, 40), (-1, -7, 1, 7)])
+def test_uneven_splits_of_square_frames(n, axial_first, crop):
+    import paper_2003_08960_gb300 as ss
+    nl = 16
+    f = _frames((n, n, nl), n)
+    lam = synth.interferograms.sweep_wavelengths(800e-9, 850e-9, nl)
+    window = crop and (crop[0] % n, crop[1] % n, crop[2], crop[3])
+    plan = ss.Plan(n, n, nl, 20e-6, 0.3, lam, window=window, flags=ss.SSOCT_FLAG_AXIAL_FIRST if axial_first else 0)
+    vol, cplx = plan.reconstruct(torch.from_numpy(f.view(np.int16)).cuda(), complex_out=True)
+    plan.sync()
+    full = oracle.reconstruct(f, 20e-6, 0.3, lam, method="fft")
+    x0, y0, wx, wy = window or (0, 0, n, n)
+    ref = full[:, y0:y0 + wy, x0:x0 + wx]
+    rms = float(np.sqrt(np.mean(oracle.intensity(full))))
+    err = cplx.cpu().numpy().astype(np.complex128) - ref
+    assert np.sqrt(np.mean(oracle.intensity(err))) <= TOL * rms
+    e = TOL * rms * np.sqrt(ref.size)
+    assert np.all(np.abs(vol.cpu().numpy().astype(np.float64) - oracle.intensity(ref)) <= 2 * e * np.abs(ref) + e * e)
+
+
 @pytest.mark.parametrize("window", [None, (100, 40, 301, 222)])
 def test_aberration_path_from_any_alignment(window):
     import paper_2003_08960_gb300 as ss
