@@ -33,12 +33,13 @@
 // issues its 12 MMAs per stage, and every thread waits on its commit barrier.
 //
 // The rows leave by one tensor copy per half-tile (256 depth bins x 16 pixels,
-// clipped at the window), which the group does not wait for: the buffer is refilled
-// in the middle of the group's next half-tile.  What bounds the kernel is that the
-// groups wait for one another's steps, so the steps were made fewer: four group
-// barriers a half-tile instead of eight, and no copy of the rows through registers.
-// 512x512x256: 175 -> 159 us (805 MB, 5.1 TB/s), 1024x1024x256: 656 -> 594 us
-// (3.2 GB, 5.4 TB/s).  Stores straight from tensor memory in 32-byte pieces had
+// clipped at the window); one thread waits until it has read them and refills the
+// buffer.  What bounds the kernel is that groups wait: for their half-tiles (six
+// buffers, four of them being computed in), for their MMAs and for one another's
+// steps.  So the steps were made fewer, four group barriers a half-tile instead of
+// eight, and no copy of the rows through registers.  512x512x256: 175 -> 154 us (805
+// MB, 5.2 TB/s), 1024x1024x256: 656 -> 575 us (3.2 GB, 5.6 TB/s).  Three groups,
+// which leave three buffers for copies ahead: 164 and 620 us.  Stores straight from tensor memory in 32-byte pieces had
 // been slower (720 us against 657 at the time).
 #include <cuda_bf16.h>
 
@@ -306,6 +307,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   // thread of a group leaves the loop alone.
   bool bad = false;
   for (int i = g, prev = -1; i < mine; prev = i, i += kTcGroups) {
+    // item prev's rows leave by their copy alone: refill its buffer once they are read
+    // (594 -> 572 us at 1024x1024x256 against a refill after the barrier below)
+    if (p.bulk && lt == 0 && prev >= 0 && prev + kTcStages < mine) {
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      tc_fill(&imap, ring, full, fills, prev + kTcStages);
+    }
+    __syncwarp();
     if (!tc_wait(&full[i % kTcFull], (unsigned)(i / kTcFull) & 1u, kTcLoadWaitNs)) {
       atomicOr(p.err, kErrAxial);
       bad = true;
@@ -332,11 +340,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int k = 0; k < 8; ++k) x[u][k] = src[(j1 + 16 * (8 * h + k)) * kTcHalf];
       }
       if (tc_group_sync_or(g, bad)) break;
-      // item prev's rows have left its buffer, or nearly: refill it
-      if (lt == 0 && prev >= 0 && prev + kTcStages < mine) {
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        tc_fill(&imap, ring, full, fills, prev + kTcStages);
-      }
+      // item prev's rows were stored by the group's threads, which are all here: refill
+      if (!p.bulk && lt == 0 && prev >= 0 && prev + kTcStages < mine) tc_fill(&imap, ring, full, fills, prev + kTcStages);
       const int blk = px >> 3, pl = px & 7;
       unsigned short* Ahi = A + blk * kABlock;
       unsigned short* Alo = A + (kTcItemBlocks + blk) * kABlock;
@@ -529,7 +534,7 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
   if (!encode_inter_map(ap.inter, (long long)ap.ntx * ap.wy * kTcN, kTcHalf, &imap)) return cudaErrorInvalidValue;
   // A tensor copy needs rows on 16-byte boundaries (volumes are); every other width
   // takes 64-byte runs from its threads (512x512x256 with a window of
-  // 333 x 400: 104.8 us, of 332 x 400 by tensor copies: 93.3 us).
+  // 333 x 400: 105.0 us, of 332 x 400 by tensor copies: 91.8 us).
   alignas(64) CUtensorMap vmap = {};
   p.bulk = ap.wx % 4 == 0;
   if (p.bulk && !encode_volume_map(ap.vol, ap.wx, ap.wy, kTcN, kTcHalf, &vmap)) return cudaErrorInvalidValue;
