@@ -868,7 +868,7 @@ def _batched(args, ss, torch, synth, w_1024, frames_1024, stream, steps=10):
             "ms_separate": ms_sep, "Gvoxel_per_s_separate": voxels / (ms_sep * 1e-3) / 1e9,
             "lanes": best, "ms_by_lanes": lanes, "graph_captures": captures,
             "form": "one CUDA graph launch per batch, volume i on stream lane i mod lanes; "
-                    "384/640/768 frames take the two-pass lateral path"}
+                    "every frame size on the persistent lateral kernel"}
 
 
 # sources every kernel is built from besides its own .cu file

@@ -104,10 +104,11 @@ typedef struct {
  *   nx, ny     frame size (pixels).  The persistent lateral kernel compiles
  *              nx, ny in {64, 128, 256, 384, 512, 640, 768, 1024} (square),
  *              plus (128, 64) and (64, 128).  Any other pair from that set
- *              (mixed radix 2/3/5) takes a two-pass lateral path
- *              (row pass, column pass through a frame buffer in the
- *              workspace); such plans do not offer ssoct_reconstruct_sliding
- *              or ssoct_reconstruct_frames_noalloc (EUNSUPPORTED there).
+ *              (mixed radix 2/3/5) keeps a frame buffer in the workspace,
+ *              for a row pass and a column pass or, from 2.5 million voxels
+ *              on, as the persistent kernel's scratch ring; such plans do
+ *              not offer ssoct_reconstruct_sliding or
+ *              ssoct_reconstruct_frames_noalloc (EUNSUPPORTED there).
  *   nlambda    frames per sweep = depth bins, N_z of Eq. 3 / the gate of Eq. 7.
  *              The library is compiled for {16, 32, 64, 96, 128, 160, 200, 256, 512}.
  *   pitch_m    camera pixel pitch d > 0.

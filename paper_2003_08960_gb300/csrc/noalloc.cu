@@ -12,8 +12,9 @@
 //
 // The array holds the plan's tables, the L2 scratch ring and work counters of
 // the lateral kernel, and the sweep-axis intermediate: the tables and counters
-// where a plan workspace has them, then the ring and the intermediate.  It has a fixed size (kNoAllocBytes), and every GPU that loads
-// the library keeps it until the process exits.  All calls share it and it keeps
+// where a plan workspace has them, then the ring and the intermediate.  It has a
+// fixed size (kNoAllocBytes), and every GPU that loads the library keeps it until
+// the process exits.  All calls share it and it keeps
 // the last call's contents: each call rewrites the tables and zeroes the
 // counters before its kernels run, and calls that overlap on the GPU (different
 // streams, or different host threads) race on it.

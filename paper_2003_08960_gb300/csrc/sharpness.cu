@@ -8,7 +8,7 @@
 //   rows    u_t = Eq. 5 resample of frame t;  row DFT (+) of c P u_t      -> F[t][y][x]
 //   columns column DFT (+), window crop                                  -> sweep-axis intermediate
 //   axial   Eq. 7 over t, P_v = |K|^2 |V~_v|^2                            -> volume
-//   sums    S1 = sum P_v, S2 = sum P_v^2 (FP64); L = -S2 / S1^2
+//   sums    S1 = sum P_v, S2 = sum P_v^2 (pairs of floats, FP64 between blocks); L = -S2 / S1^2
 // Adjoint (W = 2 |K|^2 dL/dP V~, dL/dP = -2 P / S1^2 + 2 S2 / S1^3):
 //   axial   V~ recomputed, W formed, sum_q W_q exp(+2 pi i q t / N)      -> intermediate (in place)
 //   columns zero outside the window, column DFT (-)                      -> F[t][y][x]

@@ -180,7 +180,8 @@ struct LateralSchedule {
 // slot.  Measured lateral times, paper order, against lags of 0.7 x 600 items
 // with four slots of slack: 256 x 256 x 512 353 -> 203 us, 512 x 512 x 256
 // 476 -> 347, 384 x 384 x 96 142 -> 94, 640 x 640 x 160 483 -> 401, 768 x 768 x
-// 200 722 -> 675, 1024 x 1024 x 256 1328 -> 1320; 2400 items gave no more.
+// 200 722 -> 675, 1024 x 1024 x 256 1328 -> 1320; 2400 items gave no more.  (Rows of
+// 384, 640 and 768 pixels have become faster since, see row_item.)
 constexpr int kLateralItemsInFlight = 1200;
 struct LateralPick {
   int lag, slots;
@@ -302,8 +303,8 @@ struct Plan {
   size_t off_image = 0, off_ratio = 0;
   size_t off_tcb, off_wq, off_ring, off_scratch, off_inter, ws_bytes;
   size_t off_cp = 0, off_F = 0, off_Q = 0, off_red = 0;  // SSOCT_FLAG_PUPIL regions
-  // Frame sizes the persistent lateral kernel does not compile (384, 640, 768)
-  // take the two-pass lateral path of sharpness.cu: chirp table and frame buffer.
+  // Non-square frames other than 128 x 64 and 64 x 128: chirp table and frame buffer
+  // of the two passes in sharpness.cu, which pair_queue takes as its scratch ring.
   bool generic = false;
   size_t off_cg = 0;
   // SSOCT_FLAG_AXIAL_FIRST: Eq. 5 + Eq. 7 first (half spectrum of the real

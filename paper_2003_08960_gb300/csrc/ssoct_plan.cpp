@@ -424,12 +424,13 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     p.af_option = true;
     // Whole volumes of (nearly) the whole plane run axial-first from the start:
     // lateral + axial kernels of the paper's order against first pass + lateral,
-    // us: 256 x 256 x 256 144 / 126, 384 x 384 x 96 127 / 115, 512 x 512 x 128
-    // 241 / 217, 640 x 640 x 160 534 / 492, 768 x 768 x 200 892 / 824, 1024 x 1024
-    // x 256 1798 / 1634.  The first pass covers the whole sensor whatever the
+    // us: 256 x 256 x 64 45 / 39, x 256 140 / 122, 384 x 384 x 96 120 / 103, 512 x
+    // 512 x 128 237 / 212, 640 x 640 x 160 490 / 456, 768 x 768 x 200 868 / 786, 1024 x
+    // 1024 x 256 1812 / 1628.  The first pass covers the whole sensor whatever the
     // window, the axial kernel only the window: at three quarters of a 1024 x 1024
     // plane the two orders are equal.  Frames of up to 128 x 128 go through the
-    // small kernels at the same speed either way.
+    // small kernels at the same speed either way.  Relative error of |V|^2 against
+    // float64: 2.1e-7, paper's order 1.8e-7 (of the three cuts 6.4e-7 and 7.5e-7).
     p.axial_first = nx >= 256 && !(flags & SSOCT_FLAG_TC_AXIAL) && 8ll * p.wx * p.wy >= 7ll * nx * ny;
   }
   if (p.ra_w) p.off_xstrip = take(sizeof(StripTap) * p.xstrip.size());
