@@ -343,7 +343,8 @@ struct Plan {
   unsigned long long wait_ns = 0;
   // stage timing (ssoct_profile)
   bool profiling = false;
-  std::vector<cudaEvent_t> events;  // 3 per recorded call: start, after lateral, after axial
+  std::vector<cudaEvent_t> events;  // 3 per recorded call: start, after its first stage, after its second
+  std::vector<char> events_af;      // per recorded call: axial-first order (the axial stage is its first)
   size_t events_used = 0;
 };
 

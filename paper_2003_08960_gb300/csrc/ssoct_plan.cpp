@@ -608,6 +608,22 @@ static LateralParams lateral_params(const Plan& p, const uint16_t* frames, int r
   return lp;
 }
 
+// Three events for the next call of a profile, and the order that it runs in
+// (a plan's whole volumes and its sliding gates may run in different ones).
+static cudaError_t profile_events(Plan& p, cudaEvent_t** ev) {
+  while (p.events.size() < p.events_used + 3) {
+    cudaEvent_t x;
+    const cudaError_t e = cudaEventCreate(&x);
+    if (e != cudaSuccess) return e;
+    p.events.push_back(x);
+  }
+  p.events_af.resize(p.events_used / 3);
+  p.events_af.push_back(p.axial_first);
+  *ev = p.events.data() + p.events_used;
+  p.events_used += 3;
+  return cudaSuccess;
+}
+
 // Reset the work counters and launch the lateral kernel (with the stage events
 // of ssoct_profile); *ev receives the event slots of this call, if profiling.
 static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaStream_t s, cudaEvent_t** ev) {
@@ -626,16 +642,8 @@ static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaSt
   }
   *ev = nullptr;
   if (p.profiling) {
-    if (p.events_used + 3 > p.events.size()) {
-      for (int i = 0; i < 3; ++i) {
-        cudaEvent_t x;
-        e = cudaEventCreate(&x);
-        if (e != cudaSuccess) return cuda_fail(&p, e, "event create");
-        p.events.push_back(x);
-      }
-    }
-    *ev = p.events.data() + p.events_used;
-    p.events_used += 3;
+    e = profile_events(p, ev);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "event create");
     cudaEventRecord((*ev)[0], s);
   }
   if (p.axial_first) {
@@ -745,18 +753,10 @@ static ssoct_status sliding_update(Plan& p, cudaStream_t s, cudaEvent_t** ev_out
   p.lat_upto = p.stream_count;
   if (k == 0 && p.profiling) {
     // keep the profile's three events per call: an empty lateral interval
-    cudaEvent_t* e0 = nullptr;
-    if (p.events_used + 3 > p.events.size())
-      for (int i = 0; i < 3; ++i) {
-        cudaEvent_t x;
-        if (cudaEventCreate(&x) != cudaSuccess) return fail(&p, SSOCT_ECUDA, "event create");
-        p.events.push_back(x);
-      }
-    e0 = p.events.data() + p.events_used;
-    p.events_used += 3;
-    cudaEventRecord(e0[0], s);
-    cudaEventRecord(e0[1], s);
-    ev = e0;
+    const cudaError_t e = profile_events(p, &ev);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "event create");
+    cudaEventRecord(ev[0], s);
+    cudaEventRecord(ev[1], s);
   }
   *ev_out = ev;
   return SSOCT_OK;
@@ -950,9 +950,10 @@ ssoct_status ssoct_profile_read(ssoct_plan h, double* lateral_ms, double* axial_
     if (e != cudaSuccess) return cuda_fail(&p, e, "event elapsed");
     e = cudaEventElapsedTime(&b, p.events[i + 1], p.events[i + 2]);
     if (e != cudaSuccess) return cuda_fail(&p, e, "event elapsed");
-    // axial-first plans record the rescale-axial pass first
-    lat += p.axial_first ? b : a;
-    ax += p.axial_first ? a : b;
+    // axial-first calls record the rescale-axial pass first
+    const bool af = p.events_af[i / 3] != 0;
+    lat += af ? b : a;
+    ax += af ? a : b;
   }
   if (lateral_ms) *lateral_ms = lat;
   if (axial_ms) *axial_ms = ax;
