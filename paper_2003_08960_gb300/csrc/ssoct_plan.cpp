@@ -501,6 +501,7 @@ ssoct_status ssoct_set_workspace(ssoct_plan h, void* dev_ptr, size_t bytes) {
   p.ws = ws;
   p.stream_count = 0;
   p.lat_upto = -1;
+  p.xs_valid = false;  // the running xy cut lies in the workspace
   if (p.flags & SSOCT_FLAG_PUPIL) {
     std::vector<float4> cis;
     pupil_cis_table(cis);
@@ -543,6 +544,7 @@ ssoct_status ssoct_push_frames(ssoct_plan h, const uint16_t* frames, int n, int 
       p.ring_head = 0;
       p.stream_count = 0;
       p.lat_upto = -1;
+      p.xs_valid = false;  // stream positions restart, so it could pass for the new gate's
       st = SSOCT_EDROPPED;
     }
     p.next_seq = first_seq + n;
