@@ -122,6 +122,13 @@ extern "C" ssoct_status ssoct_batch_run(ssoct_batch b, const uint16_t* const* fr
     b->vols.assign(vol_dev, vol_dev + n);
     ++b->captures;
   }
+  // every launch overwrites the plans' intermediates, a relaunch as well as the
+  // first run: what their sliding gates keep there is gone
+  for (ssoct_plan h : b->plans) {
+    Plan& p = plan_of(h);
+    p.lat_upto = -1;
+    p.xs_valid = false;
+  }
   const cudaError_t e = cudaGraphLaunch(b->exec, s);
   if (e != cudaSuccess) return batch_fail(b, SSOCT_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
   return SSOCT_OK;
