@@ -342,7 +342,7 @@ SSOCT_API ssoct_status ssoct_batch_create(const ssoct_plan* plans, int n, int la
  * work already on `stream`; returns without waiting.  The first call on a set
  * of pointers captures all plans' kernels into a graph (on its lanes); later
  * calls on the same pointers relaunch it (one cudaGraphLaunch).  Different
- * pointers recapture. */
+ * pointers, and plans given another workspace or tuned since, recapture. */
 SSOCT_API ssoct_status ssoct_batch_run(ssoct_batch b, const uint16_t* const* frames_dev, float* const* vol_dev,
                                        void* stream);
 

@@ -2,13 +2,28 @@
 // as one CUDA graph.  The first run on a set of frame / volume pointers captures
 // every plan's kernels (lateral pass, axial pass), volume i on lane (stream)
 // i mod lanes; later runs on the same pointers relaunch the instantiated graph
-// with one call.  One lane runs the volumes back to back; more lanes let a
+// with one call, as long as no plan has been given another workspace or been
+// tuned to another form.  One lane runs the volumes back to back; more lanes let a
 // volume's kernels overlap another's, which pays off only where kernels leave
 // SMs idle (the persistent lateral kernel takes every SM).
 #include <string>
 #include <vector>
 
 #include "ssoct_internal.h"
+
+namespace ssoct {
+// What of a plan its captured kernels depend on.
+struct BatchForm {
+  const char* ws;
+  int lag, slots;
+  bool axial_first, use_tc;
+  explicit BatchForm(const Plan& p)
+      : ws(p.ws), lag(p.sch.lag), slots(p.sch.slots), axial_first(p.axial_first), use_tc(p.use_tc) {}
+  bool operator==(const BatchForm& o) const {
+    return ws == o.ws && lag == o.lag && slots == o.slots && axial_first == o.axial_first && use_tc == o.use_tc;
+  }
+};
+}  // namespace ssoct
 
 struct ssoct_batch_s {
   std::vector<ssoct_plan> plans;
@@ -20,6 +35,7 @@ struct ssoct_batch_s {
   cudaGraphExec_t exec = nullptr;
   std::vector<const uint16_t*> frames;  // pointers the graph was captured with
   std::vector<float*> vols;
+  std::vector<ssoct::BatchForm> forms;  // and the plans' workspaces and forms then
   int captures = 0;
   std::string last_error;
 };
@@ -88,7 +104,8 @@ extern "C" ssoct_status ssoct_batch_run(ssoct_batch b, const uint16_t* const* fr
   }
   cudaStream_t s = (cudaStream_t)stream;
   bool same = b->exec != nullptr;
-  for (int i = 0; same && i < n; ++i) same = b->frames[i] == frames_dev[i] && b->vols[i] == vol_dev[i];
+  for (int i = 0; same && i < n; ++i)
+    same = b->frames[i] == frames_dev[i] && b->vols[i] == vol_dev[i] && b->forms[i] == BatchForm(plan_of(b->plans[i]));
   if (!same) {
     drop_graph(b);
     cudaStream_t o = b->origin;
@@ -120,6 +137,8 @@ extern "C" ssoct_status ssoct_batch_run(ssoct_batch b, const uint16_t* const* fr
     }
     b->frames.assign(frames_dev, frames_dev + n);
     b->vols.assign(vol_dev, vol_dev + n);
+    b->forms.clear();
+    for (ssoct_plan h : b->plans) b->forms.emplace_back(plan_of(h));
     ++b->captures;
   }
   // every launch overwrites the plans' intermediates, a relaunch as well as the

@@ -39,3 +39,22 @@ def test_batch_relaunch_between_gates():
     a, b = plan.reconstruct_sliding(), ref.reconstruct_sliding()
     torch.cuda.synchronize()
     assert torch.equal(a, b)
+
+
+def test_batch_follows_a_new_workspace():
+    import paper_2003_08960_gb300 as ss
+    frames = _frames(5)
+    plan = _plan(ss)
+    vol = plan.empty_volume()[0]
+    batch = ss.Batch([plan])
+    batch.run([frames], [vol])
+    batch.sync()
+    first = vol.clone()
+    moved = torch.zeros(plan.info.workspace_bytes, dtype=torch.uint8, device="cuda")
+    assert ss.ssoct_set_workspace(plan.handle, moved.data_ptr(), moved.numel()) == ss.SSOCT_OK
+    batch.run([frames], [vol])
+    batch.sync()
+    assert batch.captures == 2 and torch.equal(vol, first)
+    batch.run([frames], [vol])
+    batch.sync()
+    assert batch.captures == 2
