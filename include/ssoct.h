@@ -229,7 +229,9 @@ SSOCT_API ssoct_status ssoct_set_pupil(ssoct_plan plan, const double* coeffs, in
  * receives L, dL/dz (per metre, at the z of ssoct_set_pupil) and
  * dL/dc_1 .. dL/dc_15.  Uses the plan's sweep-axis intermediate (like the
  * reconstruct calls, it invalidates the sliding-gate state).  Synchronises
- * `stream`.  ENOTREADY before ssoct_set_pupil. */
+ * `stream`.  ENOTREADY before ssoct_set_pupil.  ETIMEOUT if a kernel gave up
+ * waiting: out_host is then untouched, vol_dev incomplete, and ssoct_sync does
+ * not report it again (an earlier call's failure is still ssoct_sync's). */
 SSOCT_API ssoct_status ssoct_sharpness(ssoct_plan plan, const uint16_t* frames_dev, float* vol_dev,
                                        double* out_host, void* stream);
 
@@ -278,7 +280,8 @@ SSOCT_API ssoct_status ssoct_profile_read(ssoct_plan plan, double* lateral_ms, d
  * on this plan start the lateral kernel's work queue `skip` items in, so the
  * items that depend on the skipped ones can never start; every device-side wait
  * gives up after wait_limit_ns (0 = the default of 2 s), the kernels return with
- * their output incomplete, and ssoct_sync reports SSOCT_ETIMEOUT.  Nothing
+ * their output incomplete, and ssoct_sync (ssoct_sharpness itself, where it runs
+ * the queue) reports SSOCT_ETIMEOUT.  Nothing
  * faults or hangs, and the device stays usable.  skip = 0, wait_limit_ns = 0
  * restores normal operation. */
 SSOCT_API ssoct_status ssoct_inject_stall(ssoct_plan plan, unsigned skip, unsigned long long wait_limit_ns);

@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kRowThreads, 1)
       // the copies never came: the sums are incomplete, and reported so; what is
       // still in flight lands before the CTA exits
       if (tid == 0) {
-        atomicOr(err, kErrAxial);
+        atomicOr(err, kErrAdjoint);
         arrived(k);
         if (i + 1 < hi) arrived(k + 1);
       }
@@ -959,8 +959,9 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   }
   const int chunks = (pl.nl + pl.sh_tpc - 1) / pl.sh_tpc;
 
-  cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
-  if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
+  cudaError_t e = cudaSuccess;
+  unsigned* const err = &sharpness_counters(pl)->err;
+  if (!have_inter) e = rows_any(false, p, chunks, s);
   if (e == cudaSuccess && !have_inter) e = cols_any(false, p, s);
   if (e == cudaSuccess) {
     AxialParams ap = {};
@@ -973,7 +974,9 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     ap.nl = pl.nl; ap.wx = pl.wx; ap.wy = pl.wy; ap.ntx = pl.ntx;
     ap.power_scale = p.alpha2;
     ap.magnitude = 0;
-    ap.err = &((Counters*)(ws + pl.off_ctr))->err;
+    ap.err = err;
+    // after the work queue, not beside its last CTAs (512 x 512 x 128: 718 us a call, 737 beside them)
+    ap.late = have_inter ? 1 : 0;
     e = launch_axial(pl, ap, s);
   }
   const size_t nvox = (size_t)pl.nl * pl.wy * pl.wx;
@@ -990,7 +993,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
                       share.ctas <= (long long)share.bands * (chunks - 2) && rows_adj_stream_smem(pl) <= 226u * 1024u;
   if (e == cudaSuccess) e = cols_any(true, p, s);
   if (e == cudaSuccess)
-    e = stream ? rows_adj_stream_any(p, share, pl.stage_rows, &((Counters*)(ws + pl.off_ctr))->err, s)
+    e = stream ? rows_adj_stream_any(p, share, pl.stage_rows, err, s)
                : rows_any(true, p, chunks, s);
   if (e == cudaSuccess) {
     const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;

@@ -116,6 +116,7 @@ struct Counters {
 constexpr unsigned kErrTimeout = 1u;      // lateral kernel: a queue wait ran out
 constexpr unsigned kErrAxialTc = 2u;      // tensor-core axial kernel: an MMA wait ran out
 constexpr unsigned kErrAxial = 4u;        // streaming axial kernel: a stage-buffer wait ran out
+constexpr unsigned kErrAdjoint = 8u;      // adjoint row pass: a stage-buffer wait ran out
 
 // Order in which the lateral kernel takes its items.  Step s holds the row
 // items of frame s (if s < nl) and then the column items of frame s - lag (if
@@ -408,8 +409,16 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
 // Aberration path (sharpness.cu): sizes it compiles, the c P table, and the
 // forward + adjoint launches that leave loss and gradient in the FP64 block at
 // off_red ([0] S1, [1] S2, [2] loss, [3] dL/dz, [4..18] dL/dc_1..15, then the
-// two coefficients of dL/dP and a block count of the kernels).
-constexpr int kShRedDoubles = 21;
+// two coefficients of dL/dP and a block count of the kernels), followed by the
+// path's own counters and error word: its time-outs are the call's status, not
+// ssoct_sync's, and an earlier call's error word stays for ssoct_sync.
+constexpr int kShRedDoubles = 22;
+inline size_t sharpness_red_bytes(int nl) {
+  return kShRedDoubles * sizeof(double) + sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)nl;
+}
+inline Counters* sharpness_counters(const Plan& p) {
+  return (Counters*)(p.ws + p.off_red + kShRedDoubles * sizeof(double));
+}
 bool sharpness_supported(int nx, int ny, int nl);
 bool generic_lateral_supported(int nx, int ny);
 // Eq. 5 + Eq. 6 as a row pass and a column pass through the frame buffer at
@@ -419,6 +428,7 @@ void build_pupil_table(int nx, int ny, double alpha, const double* coeffs, int n
 // exp(i pi k / 128), k = 0 .. 255, as pairs of floats (re hi, re lo, im hi, im lo).
 void pupil_cis_table(std::vector<float4>& out);
 // have_inter: the sweep-axis intermediate already holds the holograms of the frames.
+// The block at off_red is zeroed by the caller.
 cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, bool have_inter, cudaStream_t s);
 cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s);
 // Dynamic shared memory of the lateral kernel for a plan (bytes).

@@ -440,7 +440,9 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     const size_t chunks = (size_t)(nlambda + p.sh_tpc - 1) / p.sh_tpc;
     p.off_cp = take(sizeof(float2) * (size_t)nx * ny);
     p.off_Q = take(sizeof(float2) * chunks * ny * nx);
-    p.off_red = take(sizeof(double) * kShRedDoubles);
+    p.off_red = take(sharpness_red_bytes(nlambda));
+    // the size limit of the no-allocation path is stated without the counters
+    beside += align_up(sharpness_red_bytes(nlambda), kAlign) - align_up(sizeof(double) * kShRedDoubles, kAlign);
   }
   p.ws_bytes = off;
   p.noalloc_bytes = off - beside;
@@ -610,6 +612,13 @@ static LateralParams lateral_params(const Plan& p, const uint16_t* frames, int r
   return lp;
 }
 
+// ssoct_inject_stall: start the ticket counter past the first items.
+static cudaError_t inject_stall(const Plan& p, Counters* ctr, cudaStream_t s) {
+  if (!p.inject_skip) return cudaSuccess;
+  const cudaError_t e = cudaMemcpyAsync(&ctr->ticket, &p.inject_skip, sizeof(unsigned), cudaMemcpyHostToDevice, s);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(s);  // the host value must outlive the copy
+}
+
 // Three events for the next call of a profile, and the order that it runs in
 // (a plan's whole volumes and its sliding gates may run in different ones).
 static cudaError_t profile_events(Plan& p, cudaEvent_t** ev) {
@@ -635,13 +644,8 @@ static ssoct_status launch_lateral_pass(Plan& p, const LateralParams& lp, cudaSt
   if (p.pair_queue || (!p.generic && !lateral_small(p)))
     e = cudaMemsetAsync(ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
-  if (p.inject_skip) {
-    // start the ticket counter past the first items (ssoct_inject_stall)
-    e = cudaMemcpyAsync(ws + p.off_ctr, &p.inject_skip, sizeof(unsigned), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return cuda_fail(&p, e, "stall injection");
-    e = cudaStreamSynchronize(s);  // the host value must outlive the copy
-    if (e != cudaSuccess) return cuda_fail(&p, e, "stall injection");
-  }
+  e = inject_stall(p, (Counters*)(ws + p.off_ctr), s);
+  if (e != cudaSuccess) return cuda_fail(&p, e, "stall injection");
   *ev = nullptr;
   if (p.profiling) {
     e = profile_events(p, ev);
@@ -907,21 +911,36 @@ ssoct_status ssoct_sharpness(ssoct_plan h, const uint16_t* frames_dev, float* vo
     if (e != cudaSuccess) return cuda_fail(&p, e, "pupil table kernel");
     p.sh_dirty = false;
   }
+  Counters* const ctr = sharpness_counters(p);
+  e = cudaMemsetAsync(p.ws + p.off_red, 0, sharpness_red_bytes(p.nl), s);
+  if (e != cudaSuccess) return cuda_fail(&p, e, "sums and counter reset");
   const bool queue = p.pupil_queue && (uintptr_t)frames_dev % 16 == 0;  // the queue's bulk copies; any frames otherwise
   if (queue) {
-    e = cudaMemsetAsync(p.ws + p.off_ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
-    if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
+    e = inject_stall(p, ctr, s);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "stall injection");
     LateralParams lp = lateral_params(p, frames_dev, 0, 0);
     lp.cp = (const float2*)(p.ws + p.off_cp);
+    lp.ctr = ctr;
+    lp.rows_done = (unsigned*)(ctr + 1);
+    lp.cols_done = lp.rows_done + p.nl;
     e = launch_lateral_pupil(p, lp, p.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(&p, e, "lateral kernel launch");
   }
   e = launch_sharpness(p, frames_dev, vol_dev, queue, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "sharpness kernels");
-  e = cudaMemcpyAsync(out_host, p.ws + p.off_red + 2 * sizeof(double), 17 * sizeof(double), cudaMemcpyDeviceToHost, s);
+  // loss and gradient with the error word behind them
+  struct {
+    double red[kShRedDoubles];
+    Counters ctr;
+  } got;
+  e = cudaMemcpyAsync(&got, p.ws + p.off_red, sizeof got, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "loss and gradient read-back");
   e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "stream synchronize");
+  if (got.ctr.err & kErrTimeout) return fail(&p, SSOCT_ETIMEOUT, "lateral kernel gave up waiting on its work queue (aberration path)");
+  if (got.ctr.err & kErrAdjoint) return fail(&p, SSOCT_ETIMEOUT, "adjoint row pass gave up waiting on its stage buffers");
+  if (got.ctr.err) return fail(&p, SSOCT_ETIMEOUT, "axial kernel gave up waiting on its stage buffers (aberration path)");
+  memcpy(out_host, got.red + 2, 17 * sizeof(double));
   return SSOCT_OK;
 }
 
