@@ -74,7 +74,8 @@ __device__ __forceinline__ void st_cg_hint(float2* a, float2 v, unsigned long lo
 // kernel before it in the stream is complete and its writes are visible, then
 // lets the next one's CTAs be placed (they wait here in turn).  A kernel's
 // lifetime so begins before its predecessor's end: what another kernel of the
-// call wrote is not read with non-coherent loads (__ldg, ldg2).
+// call wrote (pushed frames among it) is not read with non-coherent loads
+// (__ldg, ldg2), which take the plan's constant tables only.
 __device__ __forceinline__ void after_previous_kernel() {
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -114,8 +115,8 @@ inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned threads
 __device__ __forceinline__ float rescale_tap_value(const uint16_t* fr, int nx, const Tap& tx, const Tap& ty) {
   const uint16_t* r0 = fr + (size_t)ty.base * nx + tx.base;
   const uint16_t* r1 = r0 + nx;
-  const float v0 = fmaf(tx.w0, (float)__ldg(r0), tx.w1 * (float)__ldg(r0 + 1));
-  const float v1 = fmaf(tx.w0, (float)__ldg(r1), tx.w1 * (float)__ldg(r1 + 1));
+  const float v0 = fmaf(tx.w0, (float)r0[0], tx.w1 * (float)r0[1]);
+  const float v1 = fmaf(tx.w0, (float)r1[0], tx.w1 * (float)r1[1]);
   return fmaf(ty.w0, v0, ty.w1 * v1);
 }
 

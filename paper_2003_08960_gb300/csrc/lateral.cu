@@ -121,7 +121,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(SmallLat<NX, NY, C>:
     const Tap ty = ytab[y];
     cyv = ldg2(p.cy + y);
     const uint4* src = reinterpret_cast<const uint4*>(p.frames + ((size_t)((p.ring_start + f) % p.nl) * NY + lo) * NX);
-    for (int i = tid; i < (hi - lo + 1) * (NX / 8); i += T) reinterpret_cast<uint4*>(raw)[i] = __ldg(src + i);
+    for (int i = tid; i < (hi - lo + 1) * (NX / 8); i += T) reinterpret_cast<uint4*>(raw)[i] = src[i];
     __syncthreads();
     const uint16_t* r0 = raw + (ty.base - lo) * NX;
     const uint16_t* r1 = r0 + NX;
