@@ -119,7 +119,8 @@ struct ShParams {
   float2* inter;           // [wy][ntx][nl][32] sweep-axis intermediate
   float2* qpart;           // [chunks][ny][nx] partial Q
   const float* vol;        // [nl][wy][wx] P_v
-  double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15, [19] float a1, a0, [20] block count
+  double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15, [19] float a1, a0, [20] block count, [21] error word
+  const unsigned* queue_err;  // the work queue's error word, or NULL
   float sum_scale;         // power of two that keeps the squares of P_v in the float range
   int nx, ny, nl, x0, y0, wx, wy, ntx, tpc;
   int ring_start;          // frame t of the gate is frames[(ring_start + t) mod nl]
@@ -620,6 +621,9 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks,
                                                            RowsAdjShare share, int band_rows) {
   after_previous_kernel();
+  // the call reads one error word back with the loss and gradient
+  if (p.queue_err && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    atomicOr(reinterpret_cast<unsigned*>(p.red + kShRedErr), *p.queue_err);
   const int tx = grid_tx(p.nx), ry = kGradThreads / tx;
   const int x = blockIdx.x * tx + threadIdx.x % tx;
   const size_t npix = (size_t)p.nx * p.ny;
@@ -944,6 +948,7 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   p.qpart = (float2*)(ws + pl.off_Q);
   p.vol = vol;
   p.red = (double*)(ws + pl.off_red);
+  p.queue_err = have_inter ? &((const Counters*)(ws + pl.off_sctr))->err : nullptr;
   p.nx = pl.nx; p.ny = pl.ny; p.nl = pl.nl;
   p.x0 = pl.x0; p.y0 = pl.y0; p.wx = pl.wx; p.wy = pl.wy; p.ntx = pl.ntx;
   p.tpc = pl.sh_tpc;
@@ -959,9 +964,9 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   }
   const int chunks = (pl.nl + pl.sh_tpc - 1) / pl.sh_tpc;
 
-  cudaError_t e = cudaSuccess;
-  unsigned* const err = &sharpness_counters(pl)->err;
-  if (!have_inter) e = rows_any(false, p, chunks, s);
+  unsigned* const err = (unsigned*)(p.red + kShRedErr);
+  cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
+  if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
   if (e == cudaSuccess && !have_inter) e = cols_any(false, p, s);
   if (e == cudaSuccess) {
     AxialParams ap = {};
@@ -975,8 +980,6 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     ap.power_scale = p.alpha2;
     ap.magnitude = 0;
     ap.err = err;
-    // after the work queue, not beside its last CTAs (512 x 512 x 128: 718 us a call, 737 beside them)
-    ap.late = have_inter ? 1 : 0;
     e = launch_axial(pl, ap, s);
   }
   const size_t nvox = (size_t)pl.nl * pl.wy * pl.wx;

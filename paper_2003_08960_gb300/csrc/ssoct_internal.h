@@ -298,6 +298,7 @@ struct Plan {
   size_t off_twra = 0;       // twiddles of the tiled first pass's split (ra_split_n1)
   size_t off_twax = 0;       // twiddles of the axial kernels' split (ax_split_n1; off_twl where the splits agree)
   size_t off_cis = 0;        // exp(i pi k / 128) (pupil_cis_table)
+  size_t off_sctr = 0;       // the work queue's counters of the aberration path
   // host image of the workspace from off_image on (the tables but the taps), and
   // the rescale ratios lambda_t / lambda_1 in it
   std::vector<unsigned char> image;
@@ -409,16 +410,12 @@ cudaError_t launch_axial_tc(const Plan& pl, const AxialParams& ap, const unsigne
 // Aberration path (sharpness.cu): sizes it compiles, the c P table, and the
 // forward + adjoint launches that leave loss and gradient in the FP64 block at
 // off_red ([0] S1, [1] S2, [2] loss, [3] dL/dz, [4..18] dL/dc_1..15, then the
-// two coefficients of dL/dP and a block count of the kernels), followed by the
-// path's own counters and error word: its time-outs are the call's status, not
-// ssoct_sync's, and an earlier call's error word stays for ssoct_sync.
+// two coefficients of dL/dP, a block count of the kernels and, in [21], the
+// path's error word).  The path's queue has counters of its own (off_sctr): its
+// time-outs are the call's status, not ssoct_sync's, and an earlier call's error
+// word stays for ssoct_sync.
 constexpr int kShRedDoubles = 22;
-inline size_t sharpness_red_bytes(int nl) {
-  return kShRedDoubles * sizeof(double) + sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)nl;
-}
-inline Counters* sharpness_counters(const Plan& p) {
-  return (Counters*)(p.ws + p.off_red + kShRedDoubles * sizeof(double));
-}
+constexpr int kShRedErr = 21;
 bool sharpness_supported(int nx, int ny, int nl);
 bool generic_lateral_supported(int nx, int ny);
 // Eq. 5 + Eq. 6 as a row pass and a column pass through the frame buffer at
@@ -427,8 +424,8 @@ cudaError_t launch_lateral_generic(const Plan& pl, const uint16_t* frames, int r
 void build_pupil_table(int nx, int ny, double alpha, const double* coeffs, int ncoeffs, std::vector<float2>& out);
 // exp(i pi k / 128), k = 0 .. 255, as pairs of floats (re hi, re lo, im hi, im lo).
 void pupil_cis_table(std::vector<float4>& out);
-// have_inter: the sweep-axis intermediate already holds the holograms of the frames.
-// The block at off_red is zeroed by the caller.
+// have_inter: the sweep-axis intermediate already holds the holograms of the frames,
+// from the queue with the counters at off_sctr.
 cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol, bool have_inter, cudaStream_t s);
 cudaError_t launch_pupil_table(const Plan& pl, cudaStream_t s);
 // Dynamic shared memory of the lateral kernel for a plan (bytes).

@@ -365,6 +365,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.off_ytab = take(sizeof(Tap) * p.ytab.size());
   const size_t before_cis = off;
   p.off_cis = take(sizeof(float4) * 256);  // used with SSOCT_FLAG_PUPIL; every plan has its place
+  p.off_sctr = take(sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)nlambda);  // likewise
   const size_t first_table = off;
   size_t beside = off - before_cis;  // bytes that the no-allocation path's size limit leaves out
   p.off_cx = take(sizeof(float2) * nx);
@@ -440,9 +441,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     const size_t chunks = (size_t)(nlambda + p.sh_tpc - 1) / p.sh_tpc;
     p.off_cp = take(sizeof(float2) * (size_t)nx * ny);
     p.off_Q = take(sizeof(float2) * chunks * ny * nx);
-    p.off_red = take(sharpness_red_bytes(nlambda));
-    // the size limit of the no-allocation path is stated without the counters
-    beside += align_up(sharpness_red_bytes(nlambda), kAlign) - align_up(sizeof(double) * kShRedDoubles, kAlign);
+    p.off_red = take(sizeof(double) * kShRedDoubles);
   }
   p.ws_bytes = off;
   p.noalloc_bytes = off - beside;
@@ -911,11 +910,11 @@ ssoct_status ssoct_sharpness(ssoct_plan h, const uint16_t* frames_dev, float* vo
     if (e != cudaSuccess) return cuda_fail(&p, e, "pupil table kernel");
     p.sh_dirty = false;
   }
-  Counters* const ctr = sharpness_counters(p);
-  e = cudaMemsetAsync(p.ws + p.off_red, 0, sharpness_red_bytes(p.nl), s);
-  if (e != cudaSuccess) return cuda_fail(&p, e, "sums and counter reset");
   const bool queue = p.pupil_queue && (uintptr_t)frames_dev % 16 == 0;  // the queue's bulk copies; any frames otherwise
   if (queue) {
+    Counters* const ctr = (Counters*)(p.ws + p.off_sctr);
+    e = cudaMemsetAsync(ctr, 0, sizeof(Counters) + 2 * sizeof(unsigned) * (size_t)p.nl, s);
+    if (e != cudaSuccess) return cuda_fail(&p, e, "counter reset");
     e = inject_stall(p, ctr, s);
     if (e != cudaSuccess) return cuda_fail(&p, e, "stall injection");
     LateralParams lp = lateral_params(p, frames_dev, 0, 0);
@@ -928,19 +927,17 @@ ssoct_status ssoct_sharpness(ssoct_plan h, const uint16_t* frames_dev, float* vo
   }
   e = launch_sharpness(p, frames_dev, vol_dev, queue, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "sharpness kernels");
-  // loss and gradient with the error word behind them
-  struct {
-    double red[kShRedDoubles];
-    Counters ctr;
-  } got;
-  e = cudaMemcpyAsync(&got, p.ws + p.off_red, sizeof got, cudaMemcpyDeviceToHost, s);
+  double red[kShRedDoubles];
+  e = cudaMemcpyAsync(red, p.ws + p.off_red, sizeof red, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "loss and gradient read-back");
   e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(&p, e, "stream synchronize");
-  if (got.ctr.err & kErrTimeout) return fail(&p, SSOCT_ETIMEOUT, "lateral kernel gave up waiting on its work queue (aberration path)");
-  if (got.ctr.err & kErrAdjoint) return fail(&p, SSOCT_ETIMEOUT, "adjoint row pass gave up waiting on its stage buffers");
-  if (got.ctr.err) return fail(&p, SSOCT_ETIMEOUT, "axial kernel gave up waiting on its stage buffers (aberration path)");
-  memcpy(out_host, got.red + 2, 17 * sizeof(double));
+  unsigned err;
+  memcpy(&err, red + kShRedErr, sizeof err);
+  if (err & kErrTimeout) return fail(&p, SSOCT_ETIMEOUT, "lateral kernel gave up waiting on its work queue (aberration path)");
+  if (err & kErrAdjoint) return fail(&p, SSOCT_ETIMEOUT, "adjoint row pass gave up waiting on its stage buffers");
+  if (err) return fail(&p, SSOCT_ETIMEOUT, "axial kernel gave up waiting on its stage buffers (aberration path)");
+  memcpy(out_host, red + 2, 17 * sizeof(double));
   return SSOCT_OK;
 }
 
