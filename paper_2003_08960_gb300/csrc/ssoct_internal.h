@@ -71,10 +71,14 @@ struct __align__(16) Tap {
 };
 
 // Eq. 5 along one axis: output pixel i reads the input at u = c + (i - c) s,
-// c = n / 2, by linear interpolation; a tap outside [0, n) reads 0.
+// c = n / 2, by linear interpolation; a tap outside [0, n) reads 0.  Host and
+// device build the same taps: u is written as the fused step that the device (and
+// an Arm host) would make of it, since an x86 host rounds the product too and
+// could put a base one row beside the device's, whose rows are staged in buffers
+// sized from the host's taps.
 __host__ __device__ inline Tap eq5_tap(int i, int n, double s) {
   const double c = n / 2.0;
-  const double u = c + (i - c) * s;
+  const double u = fma(i - c, s, c);
   const double fl = floor(u);
   const double a = u - fl;
   const long long i0 = (long long)fl, i1 = i0 + 1;
