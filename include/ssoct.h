@@ -143,7 +143,8 @@ SSOCT_API ssoct_status ssoct_set_workspace(ssoct_plan plan, void* dev_ptr, size_
 /* Append n frames [n][ny][nx] to the plan's ring of nlambda frames (the
  * buffered acquisition of the paper's pipeline).  frames_on_device != 0: the
  * pointer is device memory; otherwise host memory.  Copies are enqueued on
- * `stream` (one cudaMemcpyAsync per contiguous piece).  first_seq >= 0 is the
+ * `stream`, one per contiguous piece: a kernel for memory of the plan's device on
+ * a 16-byte boundary, cudaMemcpyAsync for any other.  first_seq >= 0 is the
  * camera sequence number of frames[0]: if it is not the number that follows the
  * previous push, the frames are still stored but the gate restarts with them and
  * EDROPPED is returned, so that no volume mixes frames across a drop (the paper

@@ -358,7 +358,13 @@ struct Plan {
 cudaError_t launch_lateral(const Plan& p, const LateralParams& lp, cudaStream_t s);
 cudaError_t launch_axial(const Plan& p, const AxialParams& ap, cudaStream_t s);
 cudaError_t launch_cuts(const CutsParams& cp, cudaStream_t s);
-// Device copy of a multiple of 16 bytes between 16-byte aligned addresses.
+// Device copy of a multiple of 16 bytes between 16-byte aligned addresses of the
+// current device, and the frames that a push hands to it: memory of the plan's
+// own device.  A copy call reaches more than a kernel does (another GPU's memory
+// without peer access, and a stream of a device that is not current).
+inline bool push_by_kernel(const cudaPointerAttributes& a, int device, int current, const void* frames) {
+  return a.type == cudaMemoryTypeDevice && a.device == device && current == device && (uintptr_t)frames % 16 == 0;
+}
 cudaError_t launch_copy_frames(void* dst, const void* src, size_t bytes, cudaStream_t s);
 // The three cuts of the current gate straight from the sweep-axis intermediate
 // (xy: one bin per pixel; xz, yz: the axial transform of the cut's tiles).

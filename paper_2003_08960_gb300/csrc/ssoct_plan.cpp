@@ -557,6 +557,15 @@ ssoct_status ssoct_push_frames(ssoct_plan h, const uint16_t* frames, int n, int 
     p.ring_head = (p.ring_head + skip) % p.nl;
     p.pushed += skip;
   }
+  bool by_kernel = false;
+  if (frames_on_device) {
+    cudaPointerAttributes a = {};
+    int current = -1;
+    if (cudaPointerGetAttributes(&a, frames) == cudaSuccess && cudaGetDevice(&current) == cudaSuccess)
+      by_kernel = push_by_kernel(a, p.device, current, frames);
+    else
+      cudaGetLastError();  // a pointer that CUDA does not know: the copy call judges it
+  }
   const cudaMemcpyKind kind = frames_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   cudaStream_t s = (cudaStream_t)stream;
   int done = skip;
@@ -565,9 +574,8 @@ ssoct_status ssoct_push_frames(ssoct_plan h, const uint16_t* frames, int n, int 
     char* dst = p.ws + p.off_ring + fbytes * p.ring_head;
     const char* src = (const char*)frames + fbytes * done;
     // a frame is a multiple of 16 bytes (nx is one of 64 pixels)
-    cudaError_t e = frames_on_device && (uintptr_t)src % 16 == 0
-                        ? launch_copy_frames(dst, src, fbytes * run, s)
-                        : cudaMemcpyAsync(dst, src, fbytes * run, kind, s);
+    cudaError_t e = by_kernel ? launch_copy_frames(dst, src, fbytes * run, s)
+                              : cudaMemcpyAsync(dst, src, fbytes * run, kind, s);
     if (e != cudaSuccess) return cuda_fail(&p, e, "frame copy");
     done += run;
     p.ring_head = (p.ring_head + run) % p.nl;
