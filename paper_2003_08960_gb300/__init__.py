@@ -39,6 +39,10 @@ def _check(status: int, plan=None, what: str = "") -> int:
 
 
 # ---------------------------------------------------------------- C names
+#
+# Addresses are whole numbers, 0 or None for NULL: "(address or 0) + 0" refuses the
+# bytes, strings, arrays and pointers of the host that ctypes would take for a
+# void pointer, at a third of what a conversion by C.c_void_p costs.
 
 def ssoct_create_plan(nx: int, ny: int, nlambda: int, pitch_m: float, z_m: float,
                       lambda_m: Sequence[float], window: Optional[Tuple[int, int, int, int]] = None,
@@ -74,44 +78,44 @@ def ssoct_workspace_bytes(plan):
 
 
 def ssoct_set_workspace(plan, dev_ptr: int, nbytes: int) -> int:
-    return _abi.lib().ssoct_set_workspace(plan, dev_ptr, nbytes)
+    return _abi.lib().ssoct_set_workspace(plan, (dev_ptr or 0) + 0, nbytes)
 
 
 def ssoct_push_frames(plan, frames_ptr: int, n: int, frames_on_device: bool, first_seq: int, stream: int) -> int:
-    return _abi.lib().ssoct_push_frames(plan, frames_ptr, n, int(bool(frames_on_device)),
-                                        first_seq, stream)
+    return _abi.lib().ssoct_push_frames(plan, (frames_ptr or 0) + 0, n, int(bool(frames_on_device)),
+                                        first_seq, (stream or 0) + 0)
 
 
 def ssoct_reconstruct_volume(plan, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_volume(plan, vol_ptr, complex_ptr or None,
-                                               stream)
+    return _abi.lib().ssoct_reconstruct_volume(plan, (vol_ptr or 0) + 0, (complex_ptr or 0) + 0,
+                                               (stream or 0) + 0)
 
 
 def ssoct_reconstruct_frames(plan, frames_ptr: int, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_frames(plan, frames_ptr, vol_ptr,
-                                               complex_ptr or None, stream)
+    return _abi.lib().ssoct_reconstruct_frames(plan, (frames_ptr or 0) + 0, (vol_ptr or 0) + 0,
+                                               (complex_ptr or 0) + 0, (stream or 0) + 0)
 
 
 def ssoct_reconstruct_sliding(plan, vol_ptr: int, complex_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_reconstruct_sliding(plan, vol_ptr, complex_ptr or None,
-                                                stream)
+    return _abi.lib().ssoct_reconstruct_sliding(plan, (vol_ptr or 0) + 0, (complex_ptr or 0) + 0,
+                                                (stream or 0) + 0)
 
 
 def ssoct_reconstruct_frames_noalloc(plan, frames_ptr: int, vol_ptr: int, complex_ptr: int, stream: int) -> int:
     """ssoct_reconstruct_frames without any device allocation (scratch in a fixed
     64 MiB device array inside the library); the plan needs no workspace."""
-    return _abi.lib().ssoct_reconstruct_frames_noalloc(plan, frames_ptr, vol_ptr,
-                                                       complex_ptr or None, stream)
+    return _abi.lib().ssoct_reconstruct_frames_noalloc(plan, (frames_ptr or 0) + 0, (vol_ptr or 0) + 0,
+                                                       (complex_ptr or 0) + 0, (stream or 0) + 0)
 
 
 def ssoct_get_cuts(plan, vol_ptr: int, x0: int, y0: int, z0: int, xy_ptr: int, xz_ptr: int, yz_ptr: int,
                    stream: int) -> int:
-    return _abi.lib().ssoct_get_cuts(plan, vol_ptr, x0, y0, z0, xy_ptr or None,
-                                     xz_ptr or None, yz_ptr or None, stream)
+    return _abi.lib().ssoct_get_cuts(plan, (vol_ptr or 0) + 0, x0, y0, z0, (xy_ptr or 0) + 0,
+                                     (xz_ptr or 0) + 0, (yz_ptr or 0) + 0, (stream or 0) + 0)
 
 
 def ssoct_sync(plan, stream: int) -> int:
-    return _abi.lib().ssoct_sync(plan, stream)
+    return _abi.lib().ssoct_sync(plan, (stream or 0) + 0)
 
 
 def ssoct_set_pupil(plan, coeffs: Sequence[float], z_m: float) -> int:
@@ -122,14 +126,14 @@ def ssoct_set_pupil(plan, coeffs: Sequence[float], z_m: float) -> int:
 def ssoct_sharpness(plan, frames_ptr: int, vol_ptr: int, stream: int):
     """Returns (status, out[17]): loss, dL/dz, dL/dc_1 .. dL/dc_15."""
     out = np.zeros(17, dtype=np.float64)
-    st = _abi.lib().ssoct_sharpness(plan, frames_ptr, vol_ptr,
-                                    out.ctypes.data_as(C.POINTER(C.c_double)), stream)
+    st = _abi.lib().ssoct_sharpness(plan, (frames_ptr or 0) + 0, (vol_ptr or 0) + 0,
+                                    out.ctypes.data_as(C.POINTER(C.c_double)), (stream or 0) + 0)
     return st, out
 
 
 def ssoct_sliding_cuts(plan, x0: int, y0: int, z0: int, xy_ptr: int, xz_ptr: int, yz_ptr: int, stream: int) -> int:
-    return _abi.lib().ssoct_sliding_cuts(plan, x0, y0, z0, xy_ptr or None, xz_ptr or None,
-                                         yz_ptr or None, stream)
+    return _abi.lib().ssoct_sliding_cuts(plan, x0, y0, z0, (xy_ptr or 0) + 0, (xz_ptr or 0) + 0,
+                                         (yz_ptr or 0) + 0, (stream or 0) + 0)
 
 
 def ssoct_inject_stall(plan, skip: int, wait_limit_ns: int) -> int:
