@@ -22,6 +22,7 @@
 #include <cstdio>
 #include <vector>
 
+#include "adjoint_share.h"
 #include "fft_common.cuh"
 #include "mbarrier.cuh"
 
@@ -117,7 +118,8 @@ struct ShParams {
   const float2* twl;       // [N2l][N1l], sign -
   float2* F;               // [nl][ny][nx] lateral work frames
   float2* inter;           // [wy][ntx][nl][32] sweep-axis intermediate
-  float2* qpart;           // [chunks][ny][nx] partial Q
+  float2* qpart;           // [chunks][ny][nx] partial Q, tpc frames each
+  RowsAdjShare share;      // the streamed adjoint row pass's sharing
   const float* vol;        // [nl][wy][wx] P_v
   double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15, [19] float a1, a0, [20] block count, [21] error word
   const unsigned* queue_err;  // the work queue's error word, or NULL
@@ -400,20 +402,13 @@ namespace {
 // F, the raw frame rows and the taps of Eq. 5) arrive by bulk copies into two stage
 // buffers, one pair ahead.  rows_adj_kernel's accumulators leave room for eight
 // warps per SM, which wait for each of these loads in turn.  The exchange is done
-// in place in the stage buffer.  A CTA writes its share of a band's sum to partial
-// sum (its rank among the band's CTAs).  Loss and gradient at 512 x 512 x 128 726 ->
-// 683 us, 1024 x 1024 x 64 1404 -> 1279, 768 x 768 x 64 887 -> 825, 256 x 256 x 256
-// 488 -> 427.  Column and row passes in turn over chunks of frames whose F stays in
+// in place in the stage buffer.  Partial sums are those of rows_adj_kernel, eight
+// frames in FP32 (see RowsAdjShare).  One per CTA and band instead, 27 to 432 frames
+// in one FP32 sum, would take 716 us where this takes 728 (loss and gradient at 512 x
+// 512 x 128), 1298 for 1346 at 1024 x 1024 x 64, 449 for 460 at 256 x 256 x 256;
+// parts of 16 frames in pairs of floats took 730 and 1366 in the first two.  rows_adj_kernel: 762,
+// 1404, 488.  Column and row passes in turn over chunks of frames whose F stays in
 // L2 were slower (16 to 96 MiB: 724 to 767 us at 512 x 512 x 128).
-struct RowsAdjShare {
-  int bands, nt, ctas;
-  __host__ __device__ long long pairs() const { return (long long)bands * nt; }
-  __host__ __device__ int first(int c) const { return (int)(pairs() * c / ctas); }  // first pair of CTA c
-  // CTA of pair i, and the number of partial sums of a band
-  __host__ __device__ int cta_of(int i) const { return (int)((((long long)i + 1) * ctas - 1) / pairs()); }
-  __host__ __device__ int slots(int band) const { return cta_of((band + 1) * nt - 1) - cta_of(band * nt) + 1; }
-};
-
 template <int NX>
 struct RowsAdjStage {
   static constexpr int RPI = kRowThreads / Lat<NX>::N1;
@@ -424,9 +419,21 @@ struct RowsAdjStage {
 
 constexpr unsigned long long kAdjWaitNs = 4000000000ull;  // 4 s
 
+// Zeroes the slots that two CTAs of rows_adj_stream_kernel add to, 64 KB each at
+// most, one a block.  A kernel of its own: beside the sums or in the column pass,
+// which have no registers to spare, it cost 32 and 21 us at 1024 x 1024 x 64.
+__global__ void __launch_bounds__(kRowThreads) zero_split_kernel(const __grid_constant__ ShParams p) {
+  after_previous_kernel();
+  const int c = blockIdx.x + 1;
+  if (!p.share.splits(c)) return;
+  const int i = p.share.first(c), band_px = p.ny / p.share.bands * p.nx;
+  float4* q = reinterpret_cast<float4*>(p.qpart + (size_t)p.share.slot(i) * p.ny * p.nx + (size_t)p.share.band(i) * band_px);
+  for (int k = threadIdx.x; k < band_px / 2; k += kRowThreads) q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 template <int NX>
 __global__ void __launch_bounds__(kRowThreads, 1)
-    rows_adj_stream_kernel(const __grid_constant__ ShParams p, RowsAdjShare share, int raw_rows, unsigned* err) {
+    rows_adj_stream_kernel(const __grid_constant__ ShParams p, int raw_rows, unsigned* err) {
   after_previous_kernel();
   using St = RowsAdjStage<NX>;
   constexpr int N1 = Lat<NX>::N1, N2 = Lat<NX>::N2, NI = Lat<NX>::NI, RPI = St::RPI, AS = Lat<NX>::AS;
@@ -437,6 +444,7 @@ __global__ void __launch_bounds__(kRowThreads, 1)
   const int r = tid / N1, j1 = tid % N1;
   const size_t stage_bytes = (St::bytes(raw_rows) + 127) / 128 * 128;
   const size_t taps_at = St::taps_at(raw_rows);
+  const RowsAdjShare& share = p.share;
   const int lo = share.first(blockIdx.x), hi = share.first(blockIdx.x + 1);
   // pair i into stage buffer (i - lo) mod 2, by one thread
   auto fill = [&](int i) {
@@ -525,17 +533,23 @@ __global__ void __launch_bounds__(kRowThreads, 1)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0 && i + 2 < hi) fill(i + 2);
-    const int band = i / share.nt;
-    if (i + 1 == hi || (i + 1) / share.nt != band) {
-      const int slot = (int)blockIdx.x - share.cta_of(band * share.nt);
-      float2* dst = p.qpart + ((size_t)slot * p.ny + band * RPI + r) * NX;
+    if (share.closes(i, hi)) {
+      const bool whole = share.whole(i, lo, hi);
+      float2* dst = p.qpart + ((size_t)share.slot(i) * p.ny + share.band(i) * RPI + r) * NX;
       static_for<0, NI>([&](auto I) {
         constexpr int ii = decltype(I)::value;
         const int k2 = j1 + N1 * ii;
         if (N2 % N1 == 0 || k2 < N2) {
 #pragma unroll
           for (int k1 = 0; k1 < N1; ++k1) {
-            dst[k2 + N2 * k1] = acc[ii * N1 + k1];
+            float2* d = dst + k2 + N2 * k1;
+            const float2 q = acc[ii * N1 + k1];
+            if (whole) {
+              *d = q;
+            } else {
+              atomicAdd(&d->x, q.x);
+              atomicAdd(&d->y, q.y);
+            }
             acc[ii * N1 + k1] = make_float2(0.f, 0.f);
           }
         }
@@ -618,8 +632,7 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 // clock and SM) took 98 us at 512 x 512 x 128; 31 us now (three blocks per SM; 36
 // with two, 33 with four: each thread still ends with some 35 FP64 operations).
 // The reads of Q alone would take 6.
-__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks,
-                                                           RowsAdjShare share, int band_rows) {
+__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks) {
   after_previous_kernel();
   // the call reads one error word back with the loss and gradient
   if (p.queue_err && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
@@ -632,9 +645,8 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
   for (int y = blockIdx.y * ry + threadIdx.x / tx; y < p.ny; y += gridDim.y * ry) {
     const size_t i = (size_t)y * p.nx + x;
     float qx = 0.f, lx = 0.f, qy = 0.f, ly = 0.f;
-    const int parts = band_rows ? share.slots(y / band_rows) : chunks;
 #pragma unroll 8
-    for (int c = 0; c < parts; ++c) {
+    for (int c = 0; c < chunks; ++c) {
       const float2 q = __ldcs(p.qpart + (size_t)c * npix + i);
       float e;
       qx = two_sum(qx, q.x, e);
@@ -770,14 +782,14 @@ size_t rows_adj_stream_smem(const Plan& pl) {
   return SIZE_MAX;
 }
 
-cudaError_t rows_adj_stream_any(const ShParams& p, const RowsAdjShare& share, int raw_rows, unsigned* err, cudaStream_t s) {
+cudaError_t rows_adj_stream_any(const ShParams& p, int raw_rows, unsigned* err, cudaStream_t s) {
 #define X(n)                                                                                                        \
   if (p.nx == n) {                                                                                                  \
     const size_t smem = 2 * ((RowsAdjStage<n>::bytes(raw_rows) + 127) / 128 * 128);                                 \
     const cudaError_t e = cudaFuncSetAttribute(rows_adj_stream_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                (int)smem);                                                          \
     if (e != cudaSuccess) return e;                                                                                 \
-    return launch_next(rows_adj_stream_kernel<n>, dim3(share.ctas), kRowThreads, smem, s, p, share, raw_rows, err); \
+    return launch_next(rows_adj_stream_kernel<n>, dim3(p.share.ctas), kRowThreads, smem, s, p, raw_rows, err); \
   }
   X(64) X(128) X(256) X(384) X(512) X(640) X(768) X(1024)
 #undef X
@@ -964,6 +976,13 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   }
   const int chunks = (pl.nl + pl.sh_tpc - 1) / pl.sh_tpc;
 
+  // The adjoint row pass is streamed where a CTA's share is longer than a chunk by
+  // enough (all chunks but two of a band, on average) and bulk copies can read the
+  // frames.
+  const RowsAdjShare share{pl.ny * pl.n1x / kRowThreads, pl.nl, pl.num_sms, pl.sh_tpc};
+  const bool stream = (uintptr_t)frames % 16 == 0 && share.fits() && share.pairs() >= 2ll * share.ctas &&
+                      share.ctas <= (long long)share.bands * (chunks - 2) && rows_adj_stream_smem(pl) <= 226u * 1024u;
+  if (stream) p.share = share;
   unsigned* const err = (unsigned*)(p.red + kShRedErr);
   cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
   if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
@@ -987,21 +1006,16 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     e = launch_next(sums_kernel, dim3(6 * pl.num_sms), kGradThreads, 0, s, p, nvox);
   }
   if (e == cudaSuccess) e = axial_adj_any(p, s);
-  // The adjoint row pass is streamed where every SM gets two pairs or more, the
-  // partial sums suffice (a band has at most ctas / bands + 2) and bulk copies can
-  // read the frames.
-  const int band_rows = kRowThreads / pl.n1x;
-  const RowsAdjShare share{pl.ny / band_rows, pl.nl, pl.num_sms};
-  const bool stream = (uintptr_t)frames % 16 == 0 && share.pairs() >= 2ll * share.ctas &&
-                      share.ctas <= (long long)share.bands * (chunks - 2) && rows_adj_stream_smem(pl) <= 226u * 1024u;
+  if (e == cudaSuccess && stream && p.share.ctas > 1)
+    e = launch_next(zero_split_kernel, dim3(p.share.ctas - 1), kRowThreads, 0, s, p);
   if (e == cudaSuccess) e = cols_any(true, p, s);
   if (e == cudaSuccess)
-    e = stream ? rows_adj_stream_any(p, share, pl.stage_rows, err, s)
+    e = stream ? rows_adj_stream_any(p, pl.stage_rows, err, s)
                : rows_any(true, p, chunks, s);
   if (e == cudaSuccess) {
     const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;
     const int gy = std::min((p.ny + ry - 1) / ry, std::max(1, 3 * pl.num_sms / gx));
-    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks, share, stream ? band_rows : 0);
+    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks);
   }
   return e;
 }
