@@ -10,7 +10,7 @@ namespace ssoct {
 // share is no shorter than a chunk): its slot is zeroed before the pass and takes
 // both parts by atomic additions, whose order changes nothing for two addends.
 struct RowsAdjShare {
-  int bands, nt, ctas, chunk;  // ctas 0: the pass is not streamed
+  int bands, nt, ctas, chunk;
   __host__ __device__ long long pairs() const { return (long long)bands * nt; }
   __host__ __device__ int first(int c) const { return (int)(pairs() * c / ctas); }  // first pair of CTA c
   __host__ __device__ int band(int i) const { return i / nt; }

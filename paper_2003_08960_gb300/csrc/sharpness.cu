@@ -24,6 +24,7 @@
 
 #include "adjoint_share.h"
 #include "fft_common.cuh"
+#include "float_sums.cuh"
 #include "mbarrier.cuh"
 
 namespace ssoct {
@@ -119,10 +120,8 @@ struct ShParams {
   float2* F;               // [nl][ny][nx] lateral work frames
   float2* inter;           // [wy][ntx][nl][32] sweep-axis intermediate
   float2* qpart;           // [chunks][ny][nx] partial Q, tpc frames each
-  RowsAdjShare share;      // the streamed adjoint row pass's sharing
   const float* vol;        // [nl][wy][wx] P_v
   double* red;             // [0] S1, [1] S2, [2..18] loss, dL/dz, dL/dc_1..15, [19] float a1, a0, [20] block count, [21] error word
-  const unsigned* queue_err;  // the work queue's error word, or NULL
   float sum_scale;         // power of two that keeps the squares of P_v in the float range
   int nx, ny, nl, x0, y0, wx, wy, ntx, tpc;
   int ring_start;          // frame t of the gate is frames[(ring_start + t) mod nl]
@@ -192,85 +191,83 @@ __global__ void __launch_bounds__(kLatTW<NY> * Lat<NY>::N1) cols_fwd_kernel(cons
   });
 }
 
-// s + err = a + b exactly (Knuth 1969).
-__device__ __forceinline__ float two_sum(float a, float b, float& err) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return s;
-}
-
 // S1 = sum P, S2 = sum P^2 over the volume, and from them the loss and the two
 // coefficients of dL/dP = a1 P + a0.  A pass over the volume should be bound by
 // its reads (20 us for 512 x 512 x 128); two FP64 operations and a conversion
-// per voxel at two FP64 operations per clock and SM took 240 (34 now, at six
-// blocks per SM; 41 at four, 47 at three, 41-44 at eight).  Each thread sums
-// in pairs of floats instead (two_sum; P^2 as its rounded square and the exact
-// remainder), which holds 48 bits, and the pairs meet in FP64.  P is scaled by a
-// power of two so that no square leaves the float range.
+// per voxel at two FP64 operations per clock and SM took 240.  Each thread sums in
+// expansions of floats instead (FloatSums), which meet in FP64, and the last block
+// adds the blocks' sums in a fixed order: 42 us.  Relative error of the loss against
+// exact sums of the volume at eight sizes, three scenes each: 8e-16 at most, the
+// FP64 sums' 3e-15 (their blocks met by atomics); pairs of floats, 9e-15, took 33 us.
+// P is scaled by a power of two so that no square leaves the float range.
 __global__ void __launch_bounds__(kGradThreads) sums_kernel(const __grid_constant__ ShParams p, size_t n) {
   after_previous_kernel();
-  // two independent sums per thread: one alone waits for its own additions
-  float h1[2] = {0.f, 0.f}, l1[2] = {0.f, 0.f}, h2[2] = {0.f, 0.f}, l2[2] = {0.f, 0.f};
-  auto add = [&](int k, float v) {
-    float e;
-    v *= p.sum_scale;
-    h1[k] = two_sum(h1[k], v, e);
-    l1[k] += e;
-    const float q = __fmul_rn(v, v);
-    h2[k] = two_sum(h2[k], q, e);
-    l2[k] += e + fmaf(v, v, -q);
-  };
+  FloatSums sum = {};
+  const float k = p.sum_scale;
   const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   const float4* v4 = reinterpret_cast<const float4*>(p.vol);  // the volume is 16-byte aligned
   const size_t n4 = n / 4;
 #pragma unroll 4
   for (size_t i = first; i < n4; i += stride) {
     const float4 v = __ldcs(v4 + i);
-    add(0, v.x);
-    add(1, v.y);
-    add(0, v.z);
-    add(1, v.w);
+    sum.add4(v.x * k, v.y * k, v.z * k, v.w * k);
   }
-  for (size_t i = n4 * 4 + first; i < n; i += stride) add(0, p.vol[i]);
-  // the lanes' pairs meet as pairs of floats, the warps' in FP64
-  auto join = [&](float& h, float& l, float h_o, float l_o) {
-    float e;
-    h = two_sum(h, h_o, e);
-    l += l_o + e;
-  };
-  join(h1[0], l1[0], h1[1], l1[1]);
-  join(h2[0], l2[0], h2[1], l2[1]);
+  for (size_t i = n4 * 4 + first; i < n; i += stride) sum.add4(p.vol[i] * k, 0.f, 0.f, 0.f);
   for (int o = 16; o; o >>= 1) {
-    join(h1[0], l1[0], __shfl_xor_sync(0xffffffffu, h1[0], o), __shfl_xor_sync(0xffffffffu, l1[0], o));
-    join(h2[0], l2[0], __shfl_xor_sync(0xffffffffu, h2[0], o), __shfl_xor_sync(0xffffffffu, l2[0], o));
+    auto other = [&](const FloatSum& f) {
+      return FloatSum{__shfl_xor_sync(0xffffffffu, f.h, o), __shfl_xor_sync(0xffffffffu, f.l, o),
+                      __shfl_xor_sync(0xffffffffu, f.m, o)};
+    };
+    sum.p.add(other(sum.p));
+    sum.q.add(other(sum.q));
   }
-  const double s1 = (double)h1[0] + l1[0], s2 = (double)h2[0] + l2[0];
-  __shared__ double sh[2][kGradThreads / 32];
-  if (threadIdx.x % 32 == 0) {
-    sh[0][threadIdx.x / 32] = s1;
-    sh[1][threadIdx.x / 32] = s2;
-  }
+  __shared__ double2 sh[kGradThreads / 32];
+  __shared__ bool last;
+  if (threadIdx.x % 32 == 0) sh[threadIdx.x / 32] = make_double2(sum.p.value(), sum.q.value());
   __syncthreads();
+  // the blocks' sums, in the memory of Q's partial sums (not in use before the adjoint row pass)
+  double2* const blocks = reinterpret_cast<double2*>(p.qpart);
   if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
+    double2 t = make_double2(0.0, 0.0);
     for (int w = 0; w < kGradThreads / 32; ++w) {
-      a += sh[0][w];
-      b += sh[1][w];
+      t.x += sh[w].x;
+      t.y += sh[w].y;
     }
-    const double inv = 1.0 / (double)p.sum_scale;  // a power of two: exact
-    atomicAdd(p.red + 0, a * inv);
-    atomicAdd(p.red + 1, b * inv * inv);
+    __stcg(blocks + blockIdx.x, t);
     __threadfence();
     // the last block to get here sees every sum
-    if (atomicAdd(reinterpret_cast<unsigned*>(p.red + 20), 1u) == gridDim.x - 1) {
-      __threadfence();
-      const double t1 = __ldcg(p.red + 0), t2 = __ldcg(p.red + 1);
-      float* c = reinterpret_cast<float*>(p.red + 19);
-      c[0] = (float)(-2.0 / (t1 * t1));
-      c[1] = (float)(2.0 * t2 / (t1 * t1 * t1));
-      p.red[2] = -t2 / (t1 * t1);
+    last = atomicAdd(reinterpret_cast<unsigned*>(p.red + 20), 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  double2 t = make_double2(0.0, 0.0);
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kGradThreads) {
+    const double2 v = __ldcg(blocks + b);
+    t.x += v.x;
+    t.y += v.y;
+  }
+  for (int o = 16; o; o >>= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+  }
+  __syncthreads();
+  if (threadIdx.x % 32 == 0) sh[threadIdx.x / 32] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    t = sh[0];
+    for (int w = 1; w < kGradThreads / 32; ++w) {
+      t.x += sh[w].x;
+      t.y += sh[w].y;
     }
+    const double inv = 1.0 / (double)k;  // a power of two: exact
+    const double t1 = t.x * inv, t2 = t.y * inv * inv;
+    p.red[0] = t1;
+    p.red[1] = t2;
+    float* c = reinterpret_cast<float*>(p.red + 19);
+    c[0] = (float)(-2.0 / (t1 * t1));
+    c[1] = (float)(2.0 * t2 / (t1 * t1 * t1));
+    p.red[2] = -t2 / (t1 * t1);
   }
 }
 
@@ -422,18 +419,18 @@ constexpr unsigned long long kAdjWaitNs = 4000000000ull;  // 4 s
 // Zeroes the slots that two CTAs of rows_adj_stream_kernel add to, 64 KB each at
 // most, one a block.  A kernel of its own: beside the sums or in the column pass,
 // which have no registers to spare, it cost 32 and 21 us at 1024 x 1024 x 64.
-__global__ void __launch_bounds__(kRowThreads) zero_split_kernel(const __grid_constant__ ShParams p) {
+__global__ void __launch_bounds__(kRowThreads) zero_split_kernel(const __grid_constant__ ShParams p, RowsAdjShare share) {
   after_previous_kernel();
   const int c = blockIdx.x + 1;
-  if (!p.share.splits(c)) return;
-  const int i = p.share.first(c), band_px = p.ny / p.share.bands * p.nx;
-  float4* q = reinterpret_cast<float4*>(p.qpart + (size_t)p.share.slot(i) * p.ny * p.nx + (size_t)p.share.band(i) * band_px);
+  if (!share.splits(c)) return;
+  const int i = share.first(c), band_px = p.ny / share.bands * p.nx;
+  float4* q = reinterpret_cast<float4*>(p.qpart + (size_t)share.slot(i) * p.ny * p.nx + (size_t)share.band(i) * band_px);
   for (int k = threadIdx.x; k < band_px / 2; k += kRowThreads) q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 template <int NX>
 __global__ void __launch_bounds__(kRowThreads, 1)
-    rows_adj_stream_kernel(const __grid_constant__ ShParams p, int raw_rows, unsigned* err) {
+    rows_adj_stream_kernel(const __grid_constant__ ShParams p, RowsAdjShare share, int raw_rows, unsigned* err) {
   after_previous_kernel();
   using St = RowsAdjStage<NX>;
   constexpr int N1 = Lat<NX>::N1, N2 = Lat<NX>::N2, NI = Lat<NX>::NI, RPI = St::RPI, AS = Lat<NX>::AS;
@@ -444,7 +441,6 @@ __global__ void __launch_bounds__(kRowThreads, 1)
   const int r = tid / N1, j1 = tid % N1;
   const size_t stage_bytes = (St::bytes(raw_rows) + 127) / 128 * 128;
   const size_t taps_at = St::taps_at(raw_rows);
-  const RowsAdjShare& share = p.share;
   const int lo = share.first(blockIdx.x), hi = share.first(blockIdx.x + 1);
   // pair i into stage buffer (i - lo) mod 2, by one thread
   auto fill = [&](int i) {
@@ -632,11 +628,12 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 // clock and SM) took 98 us at 512 x 512 x 128; 31 us now (three blocks per SM; 36
 // with two, 33 with four: each thread still ends with some 35 FP64 operations).
 // The reads of Q alone would take 6.
-__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks) {
+__global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks,
+                                                           const unsigned* queue_err) {
   after_previous_kernel();
   // the call reads one error word back with the loss and gradient
-  if (p.queue_err && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-    atomicOr(reinterpret_cast<unsigned*>(p.red + kShRedErr), *p.queue_err);
+  if (queue_err && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    atomicOr(reinterpret_cast<unsigned*>(p.red + kShRedErr), *queue_err);
   const int tx = grid_tx(p.nx), ry = kGradThreads / tx;
   const int x = blockIdx.x * tx + threadIdx.x % tx;
   const size_t npix = (size_t)p.nx * p.ny;
@@ -782,14 +779,14 @@ size_t rows_adj_stream_smem(const Plan& pl) {
   return SIZE_MAX;
 }
 
-cudaError_t rows_adj_stream_any(const ShParams& p, int raw_rows, unsigned* err, cudaStream_t s) {
+cudaError_t rows_adj_stream_any(const ShParams& p, const RowsAdjShare& share, int raw_rows, unsigned* err, cudaStream_t s) {
 #define X(n)                                                                                                        \
   if (p.nx == n) {                                                                                                  \
     const size_t smem = 2 * ((RowsAdjStage<n>::bytes(raw_rows) + 127) / 128 * 128);                                 \
     const cudaError_t e = cudaFuncSetAttribute(rows_adj_stream_kernel<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                (int)smem);                                                          \
     if (e != cudaSuccess) return e;                                                                                 \
-    return launch_next(rows_adj_stream_kernel<n>, dim3(p.share.ctas), kRowThreads, smem, s, p, raw_rows, err); \
+    return launch_next(rows_adj_stream_kernel<n>, dim3(share.ctas), kRowThreads, smem, s, p, share, raw_rows, err); \
   }
   X(64) X(128) X(256) X(384) X(512) X(640) X(768) X(1024)
 #undef X
@@ -960,7 +957,6 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   p.qpart = (float2*)(ws + pl.off_Q);
   p.vol = vol;
   p.red = (double*)(ws + pl.off_red);
-  p.queue_err = have_inter ? &((const Counters*)(ws + pl.off_sctr))->err : nullptr;
   p.nx = pl.nx; p.ny = pl.ny; p.nl = pl.nl;
   p.x0 = pl.x0; p.y0 = pl.y0; p.wx = pl.wx; p.wy = pl.wy; p.ntx = pl.ntx;
   p.tpc = pl.sh_tpc;
@@ -982,7 +978,6 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
   const RowsAdjShare share{pl.ny * pl.n1x / kRowThreads, pl.nl, pl.num_sms, pl.sh_tpc};
   const bool stream = (uintptr_t)frames % 16 == 0 && share.fits() && share.pairs() >= 2ll * share.ctas &&
                       share.ctas <= (long long)share.bands * (chunks - 2) && rows_adj_stream_smem(pl) <= 226u * 1024u;
-  if (stream) p.share = share;
   unsigned* const err = (unsigned*)(p.red + kShRedErr);
   cudaError_t e = cudaMemsetAsync(p.red, 0, kShRedDoubles * sizeof(double), s);
   if (e == cudaSuccess && !have_inter) e = rows_any(false, p, chunks, s);
@@ -1006,16 +1001,17 @@ cudaError_t launch_sharpness(const Plan& pl, const uint16_t* frames, float* vol,
     e = launch_next(sums_kernel, dim3(6 * pl.num_sms), kGradThreads, 0, s, p, nvox);
   }
   if (e == cudaSuccess) e = axial_adj_any(p, s);
-  if (e == cudaSuccess && stream && p.share.ctas > 1)
-    e = launch_next(zero_split_kernel, dim3(p.share.ctas - 1), kRowThreads, 0, s, p);
+  if (e == cudaSuccess && stream && share.ctas > 1)
+    e = launch_next(zero_split_kernel, dim3(share.ctas - 1), kRowThreads, 0, s, p, share);
   if (e == cudaSuccess) e = cols_any(true, p, s);
   if (e == cudaSuccess)
-    e = stream ? rows_adj_stream_any(p, pl.stage_rows, err, s)
+    e = stream ? rows_adj_stream_any(p, share, pl.stage_rows, err, s)
                : rows_any(true, p, chunks, s);
   if (e == cudaSuccess) {
     const int tx = grid_tx(p.nx), gx = p.nx / tx, ry = kGradThreads / tx;
     const int gy = std::min((p.ny + ry - 1) / ry, std::max(1, 3 * pl.num_sms / gx));
-    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks);
+    e = launch_next(grad_kernel, dim3(gx, gy), kGradThreads, 0, s, p, chunks,
+                    (const unsigned*)(have_inter ? &((const Counters*)(ws + pl.off_sctr))->err : nullptr));
   }
   return e;
 }
