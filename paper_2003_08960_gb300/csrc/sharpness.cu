@@ -26,6 +26,7 @@
 #include "fft_common.cuh"
 #include "float_sums.cuh"
 #include "mbarrier.cuh"
+#include "pupil_turn.cuh"
 
 namespace ssoct {
 namespace {
@@ -843,12 +844,11 @@ struct PupilParams {
 constexpr int kPupilRows = 8;  // rows of a block: their polynomials in x come from the first threads
 
 // c P per sensor pixel, the device twin of build_pupil_table.  The phase over pi
-// (chirp and Zernike sum, a polynomial of degree four) is evaluated and reduced
-// in float64, split into the nearest 1/128 and a remainder, and the remainder
-// turns the tabulated exponential (held to 48 bits) by its series: one rounding
-// to float32 at the end, as with the float64 sine and cosine, square root and
-// fmod per pixel that took 78 us at 512 x 512 (two FP64 operations per clock and
-// SM: about 15 per pixel now, 9 us).
+// (chirp and Zernike sum, a polynomial of degree four) is evaluated in float64,
+// split into the nearest 1/128 and a remainder, and the remainder turns the
+// tabulated exponential (cis_turn): one rounding to float32 and 2^-35, in the place
+// of the float64 sine and cosine, square root and fmod per pixel that took 78 us at
+// 512 x 512 (two FP64 operations per clock and SM: about 18 per pixel now, 11 us).
 __global__ void __launch_bounds__(256) pupil_table_kernel(const __grid_constant__ PupilParams p) {
   after_previous_kernel();
   __shared__ double row[kPupilRows][5];
@@ -870,17 +870,7 @@ __global__ void __launch_bounds__(256) pupil_table_kernel(const __grid_constant_
   for (int r = threadIdx.x / tx; r < kPupilRows && y0 + r < p.ny; r += 256 / tx) {
     const double* k = row[r];
     const double t = (((k[4] * dx + k[3]) * dx + k[2]) * dx + k[1]) * dx + k[0];
-    const double m = rint(t * 128.0);             // nearest 1/128
-    const float d = (float)(t - m * (1.0 / 128.0)) * 3.14159265f;
-    // m mod 256 selects the table entry (period 2), and the centring phase (-1)^(n + l) adds a half turn
-    const int e = ((int)(long long)m + 128 * ((x + y0 + r) & 1)) & 255;
-    const float4 w = cis[e];
-    const float d2 = d * d;
-    const float s = fmaf(d2 * d, -1.f / 6.f, d);
-    const float c1 = d2 * fmaf(d2, 1.f / 24.f, -0.5f);  // cos d - 1
-    const float re = w.x + (w.y + fmaf(w.x, c1, -w.z * s));
-    const float im = w.z + (w.w + fmaf(w.z, c1, w.x * s));
-    p.cp[(size_t)(y0 + r) * p.nx + x] = make_float2(re, im);
+    p.cp[(size_t)(y0 + r) * p.nx + x] = cis_turn(t, (x + y0 + r) & 1, cis);  // with the centring phase (-1)^(n + l)
   }
 }
 
