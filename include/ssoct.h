@@ -81,8 +81,11 @@ typedef enum {
  * gates, no no-allocation call, not with SSOCT_FLAG_TC_AXIAL (EUNSUPPORTED).
  * Plans made without the flag run whole volumes in this order too where it is
  * the faster one and they offer it (see ssoct_autotune): square frames of 256 and
- * more with a window of at least 7/8 of the plane; their sliding gates and
- * no-allocation calls keep the paper's order. */
+ * more with the whole plane for a window; their sliding gates and no-allocation
+ * calls keep the paper's order.  Both orders are FP32 throughout and round
+ * differently: relative L2 error of |V|^2 against float64 1.2e-7 to 1.9e-7 in the
+ * paper's order, 1.3e-7 to 2.3e-7 in this one; of a depth bin far below the
+ * strongest, 2.5e-6 and 1.5e-6 (1024 x 1024 x 256). */
 #define SSOCT_FLAG_AXIAL_FIRST 0x8u
 
 /* Read-only facts about a plan. */

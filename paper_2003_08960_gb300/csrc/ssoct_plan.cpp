@@ -423,16 +423,25 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   else if (!generic && p.ra_w && planes_bytes <= inter_bytes && !(flags & SSOCT_FLAG_PUPIL)) {
     p.off_aplanes = p.off_inter;
     p.af_option = true;
-    // Whole volumes of (nearly) the whole plane run axial-first from the start:
-    // lateral + axial kernels of the paper's order against first pass + lateral,
-    // us: 256 x 256 x 64 45 / 39, x 256 140 / 122, 384 x 384 x 96 120 / 103, 512 x
-    // 512 x 128 237 / 212, 640 x 640 x 160 490 / 456, 768 x 768 x 200 868 / 786, 1024 x
-    // 1024 x 256 1812 / 1628.  The first pass covers the whole sensor whatever the
-    // window, the axial kernel only the window: at three quarters of a 1024 x 1024
-    // plane the two orders are equal.  Frames of up to 128 x 128 go through the
-    // small kernels at the same speed either way.  Relative error of |V|^2 against
-    // float64: 2.1e-7, paper's order 1.8e-7 (of the three cuts 6.4e-7 and 7.5e-7).
-    p.axial_first = nx >= 256 && !(flags & SSOCT_FLAG_TC_AXIAL) && 8ll * p.wx * p.wy >= 7ll * nx * ny;
+    // Whole volumes of the whole plane run axial-first from the start: paper's order
+    // against axial-first, us a call, |V|^2 alone: 256 x 256 x 64 45 / 39, x 256
+    // 140 / 122, 384 x 384 x 96 120 / 103, 512 x 512 x 128 237 / 212, 640 x 640 x 160
+    // 490 / 456, 768 x 768 x 200 868 / 786, 1024 x 1024 x 256 1812 / 1628; with the
+    // complex volume 49 / 43, 159 / 129, 136 / 116, 279 / 240, 579 / 516, 1018 / 897,
+    // 2190 / 1903, 1024 x 1024 x 64 546 / 521.  The first pass covers the whole sensor
+    // whatever the window, and the lateral kernel's bounded stores cost more than the
+    // axial kernel's, so a cropped window can go either way: 960 x 960 of 1024 x 1024
+    // x 64 471 / 490 and 536 / 622 with the complex volume, x 256 1839 / 1781 and
+    // 2159 / 2280, 480 x 481 of 512 x 512 x 128 232 / 218 and 268 / 288, 600 x 601 of
+    // 640 x 640 x 160 525 / 532 and 609 / 684.  Frames of up to 128 x 128 go through
+    // the small kernels at the same speed either way.
+    // Relative L2 error against float64, paper's order / axial-first: |V|^2 1.7e-7 /
+    // 1.9e-7 at 384 x 384 x 96, 1.6e-7 / 2.0e-7 at 512 x 512 x 128, 1.2e-7 / 2.3e-7 at
+    // 640 x 640 x 160, 1.8e-7 / 2.0e-7 at 1024 x 1024 x 256 (large values pass the
+    // lateral transforms once here, and their rounding is not averaged over the
+    // frames); the xy cut of a weak plane there 2.5e-6 / 1.5e-6, xz and yz cuts
+    // 1.3e-7 / 3e-7; V within 5 % of each other, or less in this order.
+    p.axial_first = nx >= 256 && !(flags & SSOCT_FLAG_TC_AXIAL) && p.wx == nx && p.wy == ny;
   }
   if (p.ra_w) p.off_xstrip = take(sizeof(StripTap) * p.xstrip.size());
   if (!generic && !p.af_forced) p.off_xys = take(sizeof(float2) * (size_t)p.wy * p.ntx * kTile);
