@@ -314,6 +314,7 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
   p.sch.nl = nlambda;
   p.sch.n_row = ny / p.rows_per_item;
   p.sch.n_col = (p.wx + p.cols_per_item - 1) / p.cols_per_item;
+  p.small_rows = lateral_small_rows(p);
   // Ring slots the workspace holds (the autotuner may use them all): what the
   // default schedule asks for, within 64 MiB of L2 (1024 x 1024: eight).
   {
@@ -323,8 +324,10 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     // the ring that the no-allocation path's size limit is stated for
     p.slots_noalloc = std::min({std::max(6, (600 + items - 1) / items + 4), in_l2, std::max(6, nlambda)});
     // beyond 32 MiB the ring stays under a whole sweep's frame buffer (a short
-    // sweep of large frames would otherwise double its workspace)
-    const int most = std::max<long long>(6, std::min<long long>(in_l2, std::max<long long>(nlambda * 7 / 8, (32ll << 20) / slot_bytes)));
+    // sweep of large frames would otherwise double its workspace); frames that need
+    // no queue keep the least ring, for the queue that an injected stall runs
+    const int most = p.small_rows ? p.slots_noalloc
+                                  : std::max<long long>(6, std::min<long long>(in_l2, std::max<long long>(nlambda * 7 / 8, (32ll << 20) / slot_bytes)));
     const LateralPick pick = lateral_pick(nlambda, items, most);
     p.slots_alloc = std::max(pick.slots, p.slots_noalloc);
     p.sch.lag = pick.lag;
@@ -340,7 +343,6 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
       if (rows > st) st = rows;
     }
   p.stage_rows = st;
-  p.small_rows = lateral_small_rows(p);
   // The work queue for non-square frames, and for the chirp table of the
   // aberration path, where its staging fits and the sweep is long enough to fill
   // it; the two passes through the frame buffer otherwise.  Queue against two
