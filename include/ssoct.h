@@ -108,8 +108,9 @@ typedef struct {
  *              nx, ny in {64, 128, 256, 384, 512, 640, 768, 1024} (square),
  *              plus (128, 64) and (64, 128).  Any other pair from that set
  *              (mixed radix 2/3/5) keeps a frame buffer in the workspace,
- *              for a row pass and a column pass or, from 2.5 million voxels
- *              on, as the persistent kernel's scratch ring; such plans do
+ *              for a row pass and a column pass or, where the sweep is long
+ *              enough for it to pay (from 3.5 to 8 million voxels on, by the
+ *              lengths), as the persistent kernel's scratch ring; such plans do
  *              not offer ssoct_reconstruct_sliding or
  *              ssoct_reconstruct_frames_noalloc (EUNSUPPORTED there).
  *   nlambda    frames per sweep = depth bins, N_z of Eq. 3 / the gate of Eq. 7.

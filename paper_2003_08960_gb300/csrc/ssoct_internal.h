@@ -203,6 +203,30 @@ inline LateralPick lateral_pick(int frames, int items, int max_slots) {
   return r;
 }
 
+// Where the work queue is the faster lateral path for non-square frames, by voxels
+// of a sweep.  It saves the two passes their frame buffer, and pays some 15 us for
+// filling and draining; the two passes' row and column kernels are slower for 384,
+// 640 and 768 (the queue pays earlier there), and the queue's items of frames 64
+// pixels wide or high are short (it pays late or, with two powers of two, not at
+// all).  Two passes / queue, us a call: 512 x 256 x 32 38 / 45, x 64 88 / 83; 256 x
+// 128 x 128 41 / 45, x 256 82 / 76; 384 x 256 x 32 34.0 / 35.0, x 64 69 / 66; 640 x
+// 384 x 16 44 / 41, x 160 386 / 333; 1024 x 64 x 128 89 / 98, x 512 315 / 339; 64 x
+// 1024 x 64 49 / 57, x 200 147 / 140; 768 x 64 x 256 138 / 131.  A window moves the
+// line little (512 x 256 x 32 with 128 x 64: 29 / 31).
+inline bool pair_queue_pays(int nx, int ny, long long voxels) {
+  auto mixed = [](int n) { return (n & (n - 1)) != 0; };
+  if (nx == 64) return ny >= 512 && voxels >= 8000000;
+  if (ny == 64) return mixed(nx) && nx >= 640 && voxels >= 6200000;
+  if (mixed(nx) && mixed(ny)) return voxels >= 3500000;
+  if (mixed(nx) || mixed(ny)) return voxels >= 5000000;
+  return voxels >= (nx > ny ? 6500000 : 6000000);
+}
+// The same for the loss and gradient, where the queue replaces the forward passes
+// only: 256 x 256 x 128 267 / 276, x 200 422 / 414; 384 x 384 x 64 348 / 343; 512 x
+// 512 x 32 308 / 310, x 64 484 / 450; 640 x 640 x 16 327 / 331; 768 x 768 x 16 426 /
+// 405; 1024 x 1024 x 16 621 / 581.
+inline bool pupil_queue_pays(int nx, long long voxels) { return voxels >= (nx == 256 ? 12000000 : 8000000); }
+
 // Everything the lateral kernel (rescale + chirp + row FFT, column FFT) reads.
 struct LateralParams {
   const uint16_t* frames;  // batch frame f at frames + ((ring_start + f) % nl) * nx * ny

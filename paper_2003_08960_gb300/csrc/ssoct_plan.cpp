@@ -344,16 +344,12 @@ ssoct_status ssoct_create_plan(int nx, int ny, int nlambda, double pitch_m, doub
     }
   p.stage_rows = st;
   // The work queue for non-square frames, and for the chirp table of the
-  // aberration path, where its staging fits and the sweep is long enough to fill
-  // it; the two passes through the frame buffer otherwise.  Queue against two
-  // passes: 256 x 128 x 64 22.8 / 21.5 us, 384 x 256 x 32 29.3 / 35.1, 640 x 384 x
-  // 160 251 / 332, 1024 x 512 x 64 185 / 279, 768 x 1024 x 64 with a 301 x 401
-  // window 210 / 354; loss and gradient at 384 x 384 x 32 216 / 204, 512 x 512 x
-  // 32 270 / 283, 512 x 512 x 128 753 / 830, 1024 x 1024 x 64 1450 / 1606.
+  // aberration path, where its staging fits and it pays; the two passes through the
+  // frame buffer otherwise.
   const bool queue_fits = lateral_smem_bytes(p) <= 226u * 1024u;
   const long long voxels = (long long)nx * ny * nlambda;
-  p.pair_queue = generic && queue_fits && voxels >= 2500000;
-  p.pupil_queue = (flags & SSOCT_FLAG_PUPIL) && lateral_pupil_supported(nx, ny) && queue_fits && voxels >= 6000000;
+  p.pair_queue = generic && queue_fits && pair_queue_pays(nx, ny, voxels);
+  p.pupil_queue = (flags & SSOCT_FLAG_PUPIL) && lateral_pupil_supported(nx, ny) && queue_fits && pupil_queue_pays(nx, voxels);
   if (!generic && lateral_smem_bytes(p) > 227u * 1024u) {
     delete h;
     return SSOCT_EUNSUPPORTED;  // rescale ratio too far from 1 for the staging buffer
