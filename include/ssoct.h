@@ -183,9 +183,11 @@ SSOCT_API ssoct_status ssoct_reconstruct_frames(ssoct_plan plan, const uint16_t*
  * kernel's L2 scratch ring and counters, the sweep-axis intermediate) comes from
  * one file-scope device array of 64 MiB that every GPU loading the library keeps
  * until the process exits.  This call allocates nothing (no cudaMalloc, no
- * allocating library routine).  Plans whose workspace would exceed 64 MiB get
- * SSOCT_EUNSUPPORTED with a message saying so (e.g. 256 x 256 x 64 fits,
- * 512 x 512 x 32 does not).  The first call on a device looks up the array's
+ * allocating library routine).  Plans whose tables, one sweep of frames, least
+ * scratch ring and intermediate together exceed 64 MiB get SSOCT_EUNSUPPORTED
+ * with a message saying so (e.g. 256 x 256 x 64 fits, 512 x 512 x 32 does not;
+ * ssoct_workspace_size counts a larger ring and may be above 64 MiB for a plan that
+ * fits).  The first call on a device looks up the array's
  * device address (cudaGetSymbolAddress) and SM count; make that first call
  * before any stream capture.  Host threads may make their first calls at once
  * (the look-up is done once per device, under a lock).  The address is kept for
@@ -224,11 +226,12 @@ SSOCT_API ssoct_status ssoct_reconstruct_sliding(ssoct_plan plan, float* vol_dev
  * ones 0) and the distance z_m used by ssoct_sharpness (the plan's own z stays
  * in use for the other calls).  Needs SSOCT_FLAG_PUPIL and a workspace.  Host
  * only: the next ssoct_sharpness builds the c P table on the device (FP64
- * phases, one rounding to FP32). */
+ * phases; one rounding to FP32, and 1e-11). */
 SSOCT_API ssoct_status ssoct_set_pupil(ssoct_plan plan, const double* coeffs, int ncoeffs, double z_m);
 
 /* Sharpness of the pupil-corrected volume and its gradient, by one forward and
- * one hand-written adjoint pass (all on the device; FP64 sums).  With
+ * one hand-written adjoint pass (all on the device; sums over the volume in
+ * expansions of floats that meet in FP64, below 1e-15 of relative error).  With
  * P_v = |V_v|^2 of Eq. 7 over the window, L = - sum_v P_v^2 / (sum_v P_v)^2.
  * vol_dev [nlambda][wy][wx] (16-byte aligned) receives P.  out_host[17]
  * receives L, dL/dz (per metre, at the z of ssoct_set_pupil) and
@@ -244,7 +247,7 @@ SSOCT_API ssoct_status ssoct_sharpness(ssoct_plan plan, const uint16_t* frames_d
  * (new frames through Eq. 5 + Eq. 6 only), then only the three cuts of its
  * |V|^2 instead of the volume: xy[wy][wx] at depth bin z0 as one bin of Eq. 7
  * per pixel, xz[nlambda][wx] at row y0 and yz[nlambda][wy] at column x0 (window
- * coordinates) from Eq. 7 on the tiles that hold them.  Any output may be NULL.
+ * coordinates) from Eq. 7 on those lines alone.  Any output may be NULL.
  * While z0 stays the same from call to call, the xy cut is a running sum: the
  * call adds the new frames' holograms and subtracts those they replace (2k
  * slots read per pixel for k new frames instead of nlambda); after nlambda

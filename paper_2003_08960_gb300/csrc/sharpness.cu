@@ -8,7 +8,7 @@
 //   rows    u_t = Eq. 5 resample of frame t;  row DFT (+) of c P u_t      -> F[t][y][x]
 //   columns column DFT (+), window crop                                  -> sweep-axis intermediate
 //   axial   Eq. 7 over t, P_v = |K|^2 |V~_v|^2                            -> volume
-//   sums    S1 = sum P_v, S2 = sum P_v^2 (pairs of floats, FP64 between blocks); L = -S2 / S1^2
+//   sums    S1 = sum P_v, S2 = sum P_v^2 (expansions of floats, FP64 between blocks); L = -S2 / S1^2
 // Adjoint (W = 2 |K|^2 dL/dP V~, dL/dP = -2 P / S1^2 + 2 S2 / S1^3):
 //   axial   V~ recomputed, W formed, sum_q W_q exp(+2 pi i q t / N)      -> intermediate (in place)
 //   columns zero outside the window, column DFT (-)                      -> F[t][y][x]
@@ -626,9 +626,9 @@ __host__ __device__ constexpr int grid_tx(int nx) { return nx % 256 == 0 ? 256 :
 // and X^a and the Zernike combinations come in once per thread and per block.
 // The chunks of Q are added as pairs of floats (two_sum).  Evaluating the
 // polynomials and adding the chunks in FP64 per pixel (two FP64 operations per
-// clock and SM) took 98 us at 512 x 512 x 128; 31 us now (three blocks per SM; 36
-// with two, 33 with four: each thread still ends with some 35 FP64 operations).
-// The reads of Q alone would take 6.
+// clock and SM) took 98 us at 512 x 512 x 128; 34 us now (with three blocks per SM:
+// each thread still ends with some 35 FP64 operations).  The reads of Q alone would
+// take 6.
 __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ ShParams p, int chunks,
                                                            const unsigned* queue_err) {
   after_previous_kernel();
