@@ -402,10 +402,10 @@ namespace {
 // warps per SM, which wait for each of these loads in turn.  The exchange is done
 // in place in the stage buffer.  Partial sums are those of rows_adj_kernel, eight
 // frames in FP32 (see RowsAdjShare).  One per CTA and band instead, 27 to 432 frames
-// in one FP32 sum, would take 716 us where this takes 728 (loss and gradient at 512 x
-// 512 x 128), 1298 for 1346 at 1024 x 1024 x 64, 449 for 460 at 256 x 256 x 256;
-// parts of 16 frames in pairs of floats took 730 and 1366 in the first two.  rows_adj_kernel: 762,
-// 1404, 488.  Column and row passes in turn over chunks of frames whose F stays in
+// in one FP32 sum, took 716 us where this took 728 (loss and gradient at 512 x 512 x
+// 128), 1298 for 1346 at 1024 x 1024 x 64, 449 for 460 at 256 x 256 x 256; parts of 16
+// frames in pairs of floats 730 and 1366 in the first two; rows_adj_kernel 762, 1404
+// and 488 (each with the other kernels of its time).  Column and row passes in turn over chunks of frames whose F stays in
 // L2 were slower (16 to 96 MiB: 724 to 767 us at 512 x 512 x 128).
 template <int NX>
 struct RowsAdjStage {
@@ -418,8 +418,8 @@ struct RowsAdjStage {
 constexpr unsigned long long kAdjWaitNs = 4000000000ull;  // 4 s
 
 // Zeroes the slots that two CTAs of rows_adj_stream_kernel add to, 64 KB each at
-// most, one a block.  A kernel of its own: beside the sums or in the column pass,
-// which have no registers to spare, it cost 32 and 21 us at 1024 x 1024 x 64.
+// most, one a block.  A kernel of its own (4 us): in the column pass it cost 16 us at
+// 512 x 512 x 128 and 8 at 1024 x 1024 x 64, beside the sums 32 at the latter.
 __global__ void __launch_bounds__(kRowThreads) zero_split_kernel(const __grid_constant__ ShParams p, RowsAdjShare share) {
   after_previous_kernel();
   const int c = blockIdx.x + 1;
